@@ -293,17 +293,18 @@ plc_status plc_smooth(plc_ctx* ctx, const double* x, double* y, double radius);
 plc_status plc_log_stats(plc_ctx* ctx, const double* delta, double lo, double width, int nbins,
                          long long* counts, long long* outside, double* moments);
 
-/* FFT schedule of the FP32 transforms (PLC_MIXED contexts; an aid to
- * performance, the paper has no counterpart).  A length n = f1 f2 with a
- * register four-step form can run it with the factors (f1, f2) or with the
- * shared-memory Stockham stages (f1 = f2 = 0); every schedule computes the
- * same transform.  plc_set_fft_schedule selects one (INVALID_ARG if (f1, f2)
+/* FFT schedule of the transforms (an aid to performance, the paper has no
+ * counterpart).  A length n = f1 f2 with a register four-step form can run
+ * its FP32 transforms with the factors (f1, f2) or with the shared-memory
+ * Stockham stages (f1 = f2 = 0); FP64 fields run in 64-bit block fixed point
+ * (whichever factors are set) or, at f1 = f2 = 0, in the FP64 Stockham
+ * stages.  Every schedule computes the same transform.  plc_set_fft_schedule selects one (INVALID_ARG if (f1, f2)
  * is not offered for this n).  plc_autotune times `reps` (1..1000)
  * Hessian-vector products with each schedule offered for n, keeps the
  * fastest and returns it (f1, f2 and its time per Hv in microseconds, any
  * output may be NULL); it uses the solver work fields as scratch (and
  * allocates them on first use) and synchronises the stream.  On a PLC_FP64
- * context (Stockham only) it times nothing and returns the current
+ * context it times nothing and returns the current
  * schedule with *us_per_hv = 0. */
 plc_status plc_set_fft_schedule(plc_ctx* ctx, int f1, int f2);
 plc_status plc_autotune(plc_ctx* ctx, int reps, int* f1, int* f2, double* us_per_hv);

@@ -4,8 +4,6 @@
 #include "bias.h"
 
 namespace plc {
-template void bias_prior<double, double>(plc_ctx*, const double*, double, double*);
-template void bias_prior<double, float>(plc_ctx*, const float*, double, double*);
 template void bias_density<double, double>(plc_ctx*, const double*, const double*, double,
                                            double*, const double*, const double*, double*,
                                            const int32_t*, const double*, double, double*,
@@ -19,9 +17,5 @@ template void bias_gradient<double, double>(plc_ctx*, const double*, const doubl
 template void bias_gradient<double, float>(plc_ctx*, const double*, const double*, const double*,
                                            const float*, double*, float*, float*, float*, float*,
                                            bool);
-template void bias_cg_hv<double>(plc_ctx*, const double*, const double*, double*, const double*,
-                                 const double*, const double*, double*, double*, double*, bool);
-template void bias_hv<double>(plc_ctx*, const double*, const double*, const double*,
-                              const double*, double*, double*, double*);
 template void bias_fallback<double>(plc_ctx*, const double*, double*);
 }  // namespace plc

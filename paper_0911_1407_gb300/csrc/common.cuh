@@ -47,7 +47,7 @@ struct FftPlan {
   int tstep[kMaxStages];     // twiddle index step n / (ns * rad)
   unsigned ns_m[kMaxStages]; // fast-division multiplier for ns (0 when ns = 1)
   FastDiv nd;                // division by n
-  int f1, f2;                // FP32 register four-step factors n = f1 f2
+  int f1, f2;                // register four-step factors n = f1 f2
                              // (0 = the Stockham stages)
 };
 
@@ -233,17 +233,18 @@ __device__ __forceinline__ double unit_sin(int R, int m) {
 }
 
 // a * exp(SIGN 2 pi i m / R)
-template <typename T, int SIGN>
-__device__ __forceinline__ cpx<T> rot(cpx<T> a, int R, int m) {
-  using C = cpx<T>;
-  m %= R;
-  if (m == 0) return a;
-  if (4 * m == R) return cmul_si<SIGN>(a);
-  if (2 * m == R) return cmk<C>(-a.x, -a.y);
-  if (4 * m == 3 * R) return cmul_si<-SIGN>(a);
-  const T c = (T)unit_cos(R, m), sn = (T)SIGN * (T)unit_sin(R, m);
-  return cmk<C>(a.x * c - a.y * sn, a.x * sn + a.y * c);
-}
+template <typename T, int SIGN> struct Rot {
+  static __device__ __forceinline__ cpx<T> by(cpx<T> a, int R, int m) {
+    using C = cpx<T>;
+    m %= R;
+    if (m == 0) return a;
+    if (4 * m == R) return cmul_si<SIGN>(a);
+    if (2 * m == R) return cmk<C>(-a.x, -a.y);
+    if (4 * m == 3 * R) return cmul_si<-SIGN>(a);
+    const T c = (T)unit_cos(R, m), sn = (T)SIGN * (T)unit_sin(R, m);
+    return cmk<C>(a.x * c - a.y * sn, a.x * sn + a.y * c);
+  }
+};
 
 // In-register DFT of length R (natural order in and out).  R = 6, 12, 16 are
 // done four-step as R1 x R2 (2x3, 3x4, 4x4).
@@ -265,7 +266,7 @@ __device__ __forceinline__ void dft_small(cpx<T>* v) {
       for (int n1 = 0; n1 < R1; ++n1) a[n1] = v[R2 * n1 + n2];
       dft_small<T, SIGN, R1>(a);
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) y[k1 * R2 + n2] = rot<T, SIGN>(a[k1], R, n2 * k1);
+      for (int k1 = 0; k1 < R1; ++k1) y[k1 * R2 + n2] = Rot<T, SIGN>::by(a[k1], R, n2 * k1);
     }
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) {

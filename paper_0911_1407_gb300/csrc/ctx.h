@@ -33,9 +33,11 @@ enum Site {
 };
 extern const char* const kSiteNames[S_NSITES];
 
-// FP32 line-transform schedules with a register four-step form (passes4.cuh):
-// n = f1 f2.  The first entry for an n is the default; plc_autotune times
-// every entry for n and the Stockham form (f1 = f2 = 0).
+// Line-transform schedules with a register four-step form: n = f1 f2
+// (passes4.cuh in FP32, passesx.cuh for FP64 fields, which takes the first
+// entry of its n whichever is set).  The first entry for an n is the default;
+// plc_autotune times every FP32 entry for n and the Stockham form
+// (f1 = f2 = 0).
 struct FourStepShape {
   int n, f1, f2;
 };
@@ -68,6 +70,8 @@ struct plc_ctx {
   void* specB = nullptr;
   double2* tw64 = nullptr;
   float2* tw32 = nullptr;
+  void* twfx = nullptr;        // fixed-point twiddles (fxw, fx.cuh)
+  int* fxexp = nullptr;        // tile exponents of the fixed-point spectra (FxExps)
   void* twff = nullptr;        // float-float twiddles (ffc, ff.cuh)
   void* expff = nullptr;       // 2^(j/64), j < 64, float-float (exp_ff)
 

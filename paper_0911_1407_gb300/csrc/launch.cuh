@@ -9,6 +9,7 @@
 
 #include "passes.cuh"
 #include "passes4.cuh"
+#include "passesx.cuh"
 
 namespace plc {
 
@@ -103,6 +104,65 @@ bool run_four_step(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int
   }
 }
 
+// The FP64 passes in block fixed point (passesx.cuh).
+template <int N1, int N2, typename Pro, typename Epi, typename Fin>
+void run_pipelinex(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* done, int s0,
+                   const double* m_override) {
+  using Gm = GeoX<N1, N2>;
+  constexpr int n = Gm::N, h = n / 2 + 1;
+  fxc* A = static_cast<fxc*>(c->specA);
+  fxc* B = static_cast<fxc*>(c->specB);
+  const fxw* tw = static_cast<const fxw*>(c->twfx);
+  const double* M = m_override ? m_override : c->M64;
+  const FxExps ex = fx_exps(c->fxexp, n);
+  const dim3 gx(n / Gm::RY, n), gy(n / Gm::L, h);
+  set_smem4<kx_xf<N1, N2, Pro>>(Gm::smem_x);
+  set_smem4<kx_yf<N1, N2>>(Gm::smem_y);
+  set_smem4<kx_z<N1, N2>>(Gm::smem_z);
+  set_smem4<kx_yi<N1, N2>>(Gm::smem_y);
+  set_smem4<kx_xi<N1, N2, Epi, Fin>>(Gm::smem_x);
+  {
+    LaunchScope ls(c, Site(s0 + 0));
+    kx_xf<N1, N2, Pro><<<gx, kThreads, Gm::smem_x, c->stream>>>(pro, A, ex, tw, done);
+  }
+  {
+    LaunchScope ls(c, Site(s0 + 1));
+    kx_yf<N1, N2><<<gy, kThreads, Gm::smem_y, c->stream>>>(A, B, ex, tw, done);
+  }
+  {
+    LaunchScope ls(c, Site(s0 + 2));
+    kx_z<N1, N2><<<gy, kThreads, Gm::smem_z, c->stream>>>(B, ex, M, zero_dc, tw, done);
+  }
+  {
+    LaunchScope ls(c, Site(s0 + 3));
+    kx_yi<N1, N2><<<gy, kThreads, Gm::smem_y, c->stream>>>(B, A, ex, tw, done);
+  }
+  {
+    LaunchScope ls(c, Site(s0 + 4));
+    kx_xi<N1, N2, Epi, Fin><<<gx, kThreads, Gm::smem_x, c->stream>>>(A, ex, epi, fin, red_args(c),
+                                                                     tw, done);
+  }
+  check(cudaGetLastError(), "spectral pipeline launch");
+}
+
+// False when the context's schedule is the Stockham stages (run_pipeline then
+// takes the FP64 Stockham passes); any four-step schedule runs the default
+// factors of its length.
+template <typename Pro, typename Epi, typename Fin>
+bool run_fixed(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* done, int s0,
+               const double* m_override) {
+  if (!c->plan.f1) return false;
+  switch (c->n) {
+    case 256: run_pipelinex<16, 16>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
+    case 192: run_pipelinex<16, 12>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
+    case 128: run_pipelinex<16, 8>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
+    case 96: run_pipelinex<12, 8>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
+    case 64: run_pipelinex<8, 8>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
+    case 32: run_pipelinex<8, 4>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
+    default: return false;
+  }
+}
+
 // The five passes XF -> YF -> Z -> YI -> XI on the context's stream.
 template <typename T, typename Pro, typename Epi, typename Fin>
 void run_pipeline(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* done,
@@ -116,6 +176,8 @@ void run_pipeline(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int*
                               : (k64 ? S_XF64 : S_XF32);
   if constexpr (sizeof(T) == 4) {
     if (run_four_step<float>(c, pro, epi, fin, zero_dc, done, s0, m_override)) return;
+  } else {
+    if (run_fixed(c, pro, epi, fin, zero_dc, done, s0, m_override)) return;
   }
   const int n = c->n, h = n / 2 + 1;
   const size_t sm = G::smem_bytes(c->plan);

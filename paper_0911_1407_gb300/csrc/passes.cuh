@@ -17,9 +17,9 @@
 // step) and the epilogue fuses the pointwise tail (gradient of Sec. 3.1.2,
 // Hessian-vector product, dot products) into the last pass.
 //
-// These kernels serve FP64, and FP32 lengths (or schedules) without a
-// register four-step form (passes4.cuh); their line transform is a
-// mixed-radix Stockham FFT in shared memory.
+// These kernels serve lengths (or schedules) without a register four-step
+// form (passes4.cuh for FP32, passesx.cuh for FP64); their line transform is
+// a mixed-radix Stockham FFT in shared memory.
 //
 // Every block has all global loads of a tile in flight at once: the pure data
 // passes (YF, Z, YI) copy their tiles with cp.async straight into shared
