@@ -51,7 +51,7 @@ typedef enum {
 } plc_status;
 
 typedef enum {
-  PLC_FP64 = 0,  /* every field and FFT in double */
+  PLC_FP64 = 0,  /* every field in double, FFTs to double accuracy */
   PLC_MIXED = 1  /* FP32 FFTs and pointwise work, FP64 reductions and scalars;
                     the Newton solve keeps an FP64 master copy of s and takes
                     its stopping gradient in FP64 */

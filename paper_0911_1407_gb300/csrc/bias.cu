@@ -89,6 +89,7 @@ template <typename T, typename TC> struct Fields {
   int cg(double rtol2, int max_cg, int chunk, int first) {
     int launched = 0;
     int k = std::max(1, std::min(first, chunk));
+    precond<TC>(c, Dj, r, jac);
     read_scalars(c);
     while (!c->sc_host->done && launched < max_cg) {
       k = std::min(k, max_cg - launched);

@@ -232,7 +232,7 @@ template <typename T, typename TC> struct EpiBiasG {
   }
   __device__ __forceinline__ void cell(T st, T yt, TC Qi, T z, Acc* acc, T& gi, TC& ei, TC& di,
                                        TC& dj) const {
-    const T e = exp(st);
+    const T e = expt(st);
     const T dd = e * z;
     gi = yt + dd;
     ei = (TC)e;
@@ -402,7 +402,7 @@ void bias_cg_hv(plc_ctx* c, const TC* r, const TC* Dj, TC* p, const TC* E, const
   const int* done = &c->sc->done;
   const TC* Mb = bias_multiplier<TC>(c);
   if (jac)
-    run_pipeline<TC>(c, ProCgDirE<TC, true>{{r, Dj, (TC)c->jac_c, p, c->sc}, E}, EpiMul<TC>{Q, t},
+    run_pipeline<TC>(c, ProCgDirE<TC, true>{{r, precond_field<TC>(c, Dj), (TC)c->jac_c, p, c->sc}, E}, EpiMul<TC>{Q, t},
                      FinNone{}, 0, done, kBiasSites, Mb);
   else
     run_pipeline<TC>(c, ProCgDirE<TC, false>{{r, Dj, (TC)c->jac_c, p, c->sc}, E},

@@ -320,6 +320,11 @@ struct AccD {
   __device__ __forceinline__ void init(bool is_max) { v = is_max ? -INFINITY : 0.0; }
   __device__ __forceinline__ void add(double x) { v += x; }
   __device__ __forceinline__ void max(double x) { v = fmax(v, x); }
+  // |x| >= 0 orders as its bits do: integer comparisons (v starts below zero)
+  __device__ __forceinline__ void maxabs(double x) {
+    const long long b = __double_as_longlong(x) & 0x7fffffffffffffffll;
+    if (b > __double_as_longlong(v)) v = __longlong_as_double(b);
+  }
   __device__ __forceinline__ double get() const { return v; }
   __device__ __forceinline__ void merge(const AccD& o, bool is_max) {
     v = is_max ? fmax(v, o.v) : v + o.v;
@@ -339,6 +344,7 @@ struct AccK {
     s = t;
   }
   __device__ __forceinline__ void max(float x) { s = fmaxf(s, x); }
+  __device__ __forceinline__ void maxabs(float x) { s = fmaxf(s, x < 0.f ? -x : x); }
   __device__ __forceinline__ double get() const { return (double)s - (double)c; }
   // (s1 - c1) + (s2 - c2): the high parts by TwoSum (Knuth), the rounding
   // error folded into the compensation

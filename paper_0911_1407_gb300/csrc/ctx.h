@@ -109,7 +109,9 @@ struct plc_ctx {
   unsigned long long* hist = nullptr;
 
   // Solver work fields, each n^3 doubles, allocated on first use.
-  static constexpr int kNumWork = 13;
+  // The last one (PLC_FP64 contexts only) holds the Jacobi diagonal M^-1 of
+  // the CG in progress (precond).
+  static constexpr int kNumWork = 14, kPrecondField = 13;
   void* wf[kNumWork] = {};
   // Extra work fields of the linear-bias solve, allocated on its first use.
   static constexpr int kNumBiasWork = 12;
@@ -176,6 +178,9 @@ template <typename TC> void cg_init(plc_ctx* c, const double* b, const TC* D, TC
 // LSQ-Wiener filter start: D = nbar w, r = N - nbar w, CG scalars.
 template <typename TC> void lsq_init(plc_ctx* c, const int32_t* N, const double* w, double nbar,
                                      TC* D, TC* r, bool jac);
+// Before the iterations of an FP64 CG with Jacobi: M^-1 = 1 / (D + c) into its
+// work field and r^T M^-1 r (FP32 iterations divide: nothing to do).
+template <typename TC> void precond(plc_ctx* c, const TC* D, const TC* r, bool jac);
 // rtol2 < 0: the stopping parameters are read from the device scalars.
 template <typename TC> void cg_update(plc_ctx* c, TC* x, TC* r, const TC* p, const TC* Hp,
                                       const TC* D, bool jac, double rtol2, int max_iter);

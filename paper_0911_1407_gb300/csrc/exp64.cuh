@@ -40,9 +40,13 @@ __device__ __forceinline__ long long mul61(long long a, long long b) {
   return (fx{a} * fxk{fx_hi(b), fx_lo(b)}).v;
 }
 
+// The rare argument, out of line: inlined at every cell of an unrolled loop
+// it costs more instruction cache than the loop itself.
+static __device__ __noinline__ double exp64_far(double x) { return exp(x); }
+
 __device__ __forceinline__ double exp64(double x) {
   const unsigned top = (unsigned)__double2hiint(x) & 0x7fffffffu;
-  if (top >= 0x40400000u) return exp(x);                     // |x| >= 32 or NaN
+  if (top >= 0x40400000u) return exp64_far(x);               // |x| >= 32 or NaN
   const long long q = fx_from(x, -57).v;                     // x 2^57
   // n = round(x 64 / ln2)
   const int n = (int)(((long long)(int)(q >> 32) * 96817625 + (1ll << 44)) >> 45);

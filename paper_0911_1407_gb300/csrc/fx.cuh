@@ -211,4 +211,11 @@ __device__ __forceinline__ double fx_to_double(fx a, int E) {
       (long long)(u ? (bits | ((unsigned long long)sg & 0x8000000000000000ull)) : 0ull));
 }
 
+// The same for any E: NaN tiles, all-zero grids and values near the ends of
+// the double range (out of line: rare).
+static __device__ __noinline__ double fx_to_double_far(long long q, int E) {
+  if (E >= kFxNaN / 2) return __longlong_as_double(0x7ff8000000000000ll);
+  return q == 0 ? 0.0 : ldexp((double)q, max(E, -4000));
+}
+
 }  // namespace plc

@@ -349,6 +349,9 @@ void capture_step(plc_ctx* c, const std::vector<cudaStream_t>& st, int lv, DevCt
   TC* p = as<TC>(F[11]);
   TC* Hp = as<TC>(F[12]);
   cudaGraph_t body;
+  const long long kp = total_launches(c);
+  precond<TC>(c, as<TC>(cur.D), as<TC>(cur.r), jac);
+  const int nk_pre = (int)(total_launches(c) - kp);
   add_conditional(st[lv], h_cg, cudaGraphCondTypeWhile, 1, &body);
   capture_into(c, body, st[lv + 1], [&]() {
     const long long k0 = total_launches(c);
@@ -358,7 +361,7 @@ void capture_step(plc_ctx* c, const std::vector<cudaStream_t>& st, int lv, DevCt
     k_ctl_cg<<<1, 1, 0, c->stream>>>(t, c->sc, h_cg, nk);
     check(cudaGetLastError(), "k_ctl_cg");
   });
-  k_ctl_step<<<1, 1, 0, st[lv]>>>(t, c->sc, h_ls, h_newton, 1);
+  k_ctl_step<<<1, 1, 0, st[lv]>>>(t, c->sc, h_ls, h_newton, 1 + nk_pre);
   check(cudaGetLastError(), "k_ctl_step");
   add_conditional(st[lv], h_ls, cudaGraphCondTypeWhile, 1, &body);
   capture_into(c, body, st[lv + 1], [&]() {

@@ -35,4 +35,5 @@ template void cg_update<float>(plc_ctx*, float*, float*, const float*, const flo
 template void diag<float>(plc_ctx*, const double*, const double*, double, float*);
 template void convert<double, float>(plc_ctx*, const float*, double*);
 template void convert<float, double>(plc_ctx*, const double*, float*);
+template void precond<float>(plc_ctx*, const float*, const float*, bool);
 }  // namespace plc

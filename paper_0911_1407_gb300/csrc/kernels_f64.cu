@@ -34,4 +34,5 @@ template void cg_init<double>(plc_ctx*, const double*, const double*, double*, b
 template void cg_update<double>(plc_ctx*, double*, double*, const double*, const double*,
                                 const double*, bool, double, int);
 template void diag<double>(plc_ctx*, const double*, const double*, double, double*);
+template void precond<double>(plc_ctx*, const double*, const double*, bool);
 }  // namespace plc

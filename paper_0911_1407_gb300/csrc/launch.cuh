@@ -226,9 +226,9 @@ template <typename T> void hessvec_s(plc_ctx* c, const T* s, const T* w, double 
 template <typename T> void grad_public(plc_ctx* c, const T* s, const T* w, const int32_t* N,
                                        double nbar, T* g) {
   run_pipeline<T>(c, ProShift<T, T>{s, c->mu},
-                  EpiGrad<T, T, T, T>{s, w, N, nbar, c->mu, nullptr, g, nullptr, nullptr,
-                                      c->jac_c, 0},
-                  FinStore<6>{}, 0, nullptr, true);
+                  EpiGrad<T, T, T, T, 2>{s, w, N, nbar, c->mu, nullptr, g, nullptr, nullptr,
+                                         c->jac_c, 0},
+                  FinStore<2>{}, 0, nullptr, true);
 }
 
 template <typename T, typename TS, typename TC>
@@ -239,12 +239,13 @@ void grad_newton(plc_ctx* c, const TS* s, const double* w, const int32_t* N, dou
     // epilogue where the length has a four-step schedule
     const EpiGradFF<true> epi{s, w, N, ff(nbar), ff(c->mu), y, g, D, r, (float)c->jac_c,
                               jac ? 1 : 0, static_cast<const ff*>(c->expff)};
-    if (run_four_step<ff>(c, ProShiftFF{s, ff(c->mu)}, epi, FinGrad{}, 0, nullptr, S_GXFF)) return;
+    if (run_four_step<ff>(c, ProShiftFF{s, ff(c->mu)}, epi, FinGrad<6>{}, 0, nullptr, S_GXFF)) return;
   }
+  constexpr int NS = sizeof(TC) == 8 ? 5 : 6;
   run_pipeline<T>(c, ProShift<T, TS>{s, c->mu},
-                  EpiGrad<T, TS, double, TC>{s, w, N, nbar, c->mu, y, g, D, r, c->jac_c,
-                                             jac ? 1 : 0},
-                  FinGrad{}, 0, nullptr, true);
+                  EpiGrad<T, TS, double, TC, NS>{s, w, N, nbar, c->mu, y, g, D, r, c->jac_c,
+                                                 jac ? 1 : 0},
+                  FinGrad<NS>{}, 0, nullptr, true);
 }
 
 // The sums of the FP64 gradient of the mixed solve at an FP64 s (the
@@ -256,7 +257,7 @@ inline bool grad_sums_ff_impl(plc_ctx* c, const double* s, const double* w, cons
                               double nbar, bool jac) {
   const EpiGradFF<false> epi{s, w, N, ff(nbar), ff(c->mu), nullptr, nullptr, nullptr, nullptr,
                              (float)c->jac_c, jac ? 1 : 0, static_cast<const ff*>(c->expff)};
-  return run_four_step<ff>(c, ProShiftFF{s, ff(c->mu)}, epi, FinGrad{}, 0, nullptr, S_GXFF);
+  return run_four_step<ff>(c, ProShiftFF{s, ff(c->mu)}, epi, FinGrad<6>{}, 0, nullptr, S_GXFF);
 }
 
 template <typename T, typename TS, typename TC>
@@ -264,13 +265,20 @@ void grad_newton_g(plc_ctx* c, const TS* delta, const double* w, const int32_t* 
                    T* y, T* g, TC* D, TC* r, bool jac) {
   run_pipeline<T>(c, ProShift<T, TS>{delta, 0.0},
                   EpiGradG<T, TS, TC>{delta, w, N, nbar, y, g, D, r, c->jac_c, jac ? 1 : 0},
-                  FinGrad{}, 0, nullptr, true);
+                  FinGrad<6>{}, 0, nullptr, true);
+}
+
+// The field the CG's Jacobi products read: D for FP32, the stored M^-1
+// (precond) for FP64.
+template <typename T> inline const T* precond_field(const plc_ctx* c, const T* D) {
+  if constexpr (sizeof(T) == 8) return static_cast<const T*>(c->wf[plc_ctx::kPrecondField]);
+  else return D;
 }
 
 template <typename T> void cg_hv(plc_ctx* c, const T* r, const T* D, T* p, T* Hp, bool jac) {
   const int* done = &c->sc->done;
   if (jac)
-    run_pipeline<T>(c, ProCgDir<T, true>{r, D, (T)c->jac_c, p, c->sc},
+    run_pipeline<T>(c, ProCgDir<T, true>{r, precond_field<T>(c, D), (T)c->jac_c, p, c->sc},
                     EpiHessD<T>{D, p, Hp}, FinAlpha{}, 0, done);
   else
     run_pipeline<T>(c, ProCgDir<T, false>{r, D, (T)c->jac_c, p, c->sc},
@@ -328,15 +336,26 @@ template <typename TC> void lsq_init(plc_ctx* c, const int32_t* N, const double*
   check(cudaGetLastError(), "k_lsq_init");
 }
 
+template <typename TC> void precond(plc_ctx* c, const TC* D, const TC* r, bool jac) {
+  if constexpr (sizeof(TC) == 8) {
+    if (!jac) return;
+    LaunchScope ls(c, S_CG_INIT);
+    k_precond<TC><<<pw_blocks(c), kThreads, 0, c->stream>>>(
+        D, r, (TC)c->jac_c, static_cast<TC*>(c->wf[plc_ctx::kPrecondField]), c->n3(), red_args(c));
+    check(cudaGetLastError(), "k_precond");
+  }
+}
+
 template <typename TC> void cg_update(plc_ctx* c, TC* x, TC* r, const TC* p, const TC* Hp,
                                       const TC* D, bool jac, double rtol2, int max_iter) {
-  // one wave (4 blocks of 256 per SM at its 56 registers): 73.8 us against
-  // 77.1 with two waves at 256^3
-  const int nb = pointwise_blocks((long long)c->n3(), c->sms, 4);
+  // one wave (FP32: 4 blocks of 256 per SM at its 56 registers, 73.8 us
+  // against 77.1 with two waves at 256^3)
+    const int nb = pointwise_blocks((long long)c->n3(), c->sms, sizeof(TC) == 8 ? 3 : 4);
   LaunchScope ls(c, sizeof(TC) == 4 ? S_CG_UPDATE32 : S_CG_UPDATE64);
   if (jac)
-    k_cg_update<TC, true><<<nb, kThreads, 0, c->stream>>>(x, r, p, Hp, D, (TC)c->jac_c, c->n3(),
-                                                           red_args(c), rtol2, max_iter);
+    k_cg_update<TC, true><<<nb, kThreads, 0, c->stream>>>(x, r, p, Hp, precond_field<TC>(c, D),
+                                                           (TC)c->jac_c, c->n3(), red_args(c),
+                                                           rtol2, max_iter);
   else
     k_cg_update<TC, false><<<nb, kThreads, 0, c->stream>>>(x, r, p, Hp, D, (TC)c->jac_c, c->n3(),
                                                             red_args(c), rtol2, max_iter);

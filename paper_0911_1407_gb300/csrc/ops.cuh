@@ -12,6 +12,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "exp64.cuh"
 #include "ff.cuh"
 
 namespace plc {
@@ -45,6 +46,11 @@ __device__ __forceinline__ void st4(double* p, const V4<double>& a) {
 // needs it (a fast reciprocal for FP32; M stays a fixed positive diagonal).
 __device__ __forceinline__ float jacobi(float r, float d, float c) { return __fdividef(r, d + c); }
 __device__ __forceinline__ double jacobi(double r, double d, double c) { return r / (d + c); }
+// M^-1 r inside a CG: from D for FP32, from the stored diagonal M^-1
+// (k_precond) for FP64, whose division takes about ten operations of a pipe
+// that issues two per SM and clock.
+__device__ __forceinline__ float jprec(float r, float d, float c) { return jacobi(r, d, c); }
+__device__ __forceinline__ double jprec(double r, double m, double) { return r * m; }
 
 // ------------------------------- prologues --------------------------------
 // Every prologue has prepare(), run once per block before the element loop.
@@ -82,7 +88,7 @@ template <typename T, bool JAC> struct ProCgDir {
   // 63.0-63.3 at 8 and 61.3 at 2 for 256^3 (three loads per step)
   static constexpr int kBatch = 4;
   const T* r;
-  const T* D;
+  const T* D;          // FP64: the stored M^-1
   T c;                 // (S^-1)_ii, the prior's share of diag(H)
   T* p;
   const DevScalars* sc;
@@ -95,7 +101,7 @@ template <typename T, bool JAC> struct ProCgDir {
   }
   __device__ T operator()(size_t i) const {
     const T ri = __ldg(r + i);
-    const T zi = JAC ? jacobi(ri, __ldg(D + i), c) : ri;
+    const T zi = JAC ? jprec(ri, __ldg(D + i), c) : ri;
     const T pn = beta == (T)0 ? zi : zi + beta * __ldg(p + i);
     p[i] = pn;
     return pn;
@@ -107,7 +113,7 @@ template <typename T, bool JAC> struct ProCgDir {
     if (beta != (T)0) pv = ld4(p + i);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const T zi = JAC ? jacobi(rv.v[j], dv.v[j], c) : rv.v[j];
+      const T zi = JAC ? jprec(rv.v[j], dv.v[j], c) : rv.v[j];
       o.v[j] = beta == (T)0 ? zi : zi + beta * pv.v[j];
     }
     st4(p + i, o);
@@ -236,7 +242,7 @@ template <typename T> struct EpiHessS {
     if (w) prefetch_l2(w + i, cnt * sizeof(T));
   }
   __device__ void operator()(size_t i, T y, Acc*) const {
-    const T d = nbar * (w ? __ldg(w + i) : (T)1) * exp(__ldg(s + i));
+    const T d = nbar * (w ? __ldg(w + i) : (T)1) * expt(__ldg(s + i));
     out[i] = y + d * __ldg(v + i);
   }
   __device__ void vec4(size_t i, const V4<T>& y, Acc*) const {
@@ -244,7 +250,7 @@ template <typename T> struct EpiHessS {
     V4<T> wv{{(T)1, (T)1, (T)1, (T)1}}, o;
     if (w) wv = ld4(w + i);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) o.v[j] = y.v[j] + nbar * wv.v[j] * exp(sv.v[j]) * vv.v[j];
+    for (int j = 0; j < 4; ++j) o.v[j] = y.v[j] + nbar * wv.v[j] * expt(sv.v[j]) * vv.v[j];
     st4(out + i, o);
   }
 };
@@ -286,8 +292,10 @@ template <typename T> struct EpiHessD {
 // D = nbar w e^s and the CG start r = -g.
 // acc = { sum (s-mu) y, sum (D - N s), sum g^2, sum N s, sum N |s|,
 //         sum r M^-1 r }  with M = diag(D + c) (Jacobi) or I.
-template <typename T, typename TS, typename TW, typename TC> struct EpiGrad {
-  static constexpr int NV = 6;
+// NS: how many of the sums: 2 for the public call, 5 where k_precond takes the
+// last one (FP64 CG fields), 6 otherwise.
+template <typename T, typename TS, typename TW, typename TC, int NS> struct EpiGrad {
+  static constexpr int NV = NS;
   static constexpr unsigned MAXMASK = 0;
   using Acc = typename AccOf<T>::type;
   const TS* s;
@@ -307,16 +315,20 @@ template <typename T, typename TS, typename TW, typename TC> struct EpiGrad {
   }
   // one cell: returns g and d, accumulates the sums
   __device__ __forceinline__ void cell(T st, T wt, T ni, T y, Acc* acc, T& gi, T& d) const {
-    d = (T)nbar * wt * exp(st);
+    d = (T)nbar * wt * expt(st);
     gi = y + d - ni;
     acc[0].add((st - (T)mu) * y);
     acc[1].add(d - ni * st);
-    acc[2].add(gi * gi);
-    acc[3].add(ni * st);
-    acc[4].add(ni * (st < (T)0 ? -st : st));
-    // r^T M^-1 r in the precision of the CG fields
-    const TC gc = (TC)gi;
-    acc[5].add((T)(jac ? gc * jacobi(gc, (TC)d, (TC)c) : gc * gc));
+    if constexpr (NS > 2) {
+      acc[2].add(gi * gi);
+      acc[3].add(ni * st);
+      acc[4].add(ni * (st < (T)0 ? -st : st));
+    }
+    if constexpr (NS > 5) {
+      // r^T M^-1 r in the precision of the CG fields
+      const TC gc = (TC)gi;
+      acc[5].add((T)(jac ? gc * jacobi(gc, (TC)d, (TC)c) : gc * gc));
+    }
   }
   __device__ void operator()(size_t i, T y, Acc* acc) const {
     T gi, d;
@@ -462,12 +474,13 @@ template <int NV> struct FinStore {
 
 // After a gradient: store the sums and start CG on H xi = -g from xi = 0
 // (r = -g was written by the epilogue).  The CG tolerance and iteration cap
-// are arguments of the CG update.
-struct FinGrad {
+// are arguments of the CG update.  NS = 5: r^T M^-1 r is ||r||^2 (M = I) until
+// k_precond sets it.
+template <int NS> struct FinGrad {
   __device__ void operator()(const double* t, DevScalars* sc) const {
 #pragma unroll
-    for (int j = 0; j < 6; ++j) sc->red[j] = t[j];
-    sc->rz = t[5];
+    for (int j = 0; j < NS; ++j) sc->red[j] = t[j];
+    sc->rz = t[NS > 5 ? 5 : 2];
     sc->rr = t[2];
     sc->bnorm2 = t[2];
     sc->iter = 0;
@@ -563,11 +576,40 @@ k_cg_init(const TB* __restrict__ b, const TC* __restrict__ D, TC c, TC* __restri
   block_reduce_finish_acc<2, 0u>(acc, ra, FinCgStart{});
 }
 
+// FP64 Jacobi preconditioner of a CG solve: m = 1 / (D + c) once, so that the
+// iterations multiply, and r^T M^-1 r for its start.
+template <typename TC>
+__global__ void __launch_bounds__(kThreads)
+k_precond(const TC* __restrict__ D, const TC* __restrict__ r, TC c, TC* __restrict__ m, size_t n3,
+          RedArgs ra) {
+  typename AccOf<TC>::type acc[1];
+  acc[0].init(false);
+  const size_t step = (size_t)gridDim.x * blockDim.x * 4;
+  for (size_t i = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) * 4; i < n3; i += step) {
+    const V4<TC> dv = ld4(D + i), rv = ld4(r + i);
+    V4<TC> o;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      o.v[j] = (TC)1 / (dv.v[j] + c);
+      acc[0].add(rv.v[j] * (rv.v[j] * o.v[j]));
+    }
+    st4(m + i, o);
+  }
+  struct Fin {
+    __device__ void operator()(const double* t, DevScalars* sc) const { sc->rz = t[0]; }
+  };
+  block_reduce_finish_acc<1, 0u>(acc, ra, Fin{});
+}
+
 // x += alpha p (x = alpha p on the first step, so x needs no clearing),
 // r -= alpha H p, then r^T M^-1 r, ||r||^2 and max |x| for beta, the
 // stopping test ||r||^2 <= rtol^2 ||b||^2 and the Newton step cap.
+// Bound by HBM in FP32 (73.8 us at 256^3, 0.94 of the copy rate).  FP64: five
+// FP64 operations per cell take as long as the 56 B move, 204 us at 256^3 and
+// 41 at 128^3 (83.5 with the division and the FP64 comparison); one wave of
+// three blocks per SM, as its 78 registers allow.
 template <typename TC, bool JAC>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, sizeof(TC) == 8 ? 3 : 1)
 k_cg_update(TC* __restrict__ x, TC* __restrict__ r, const TC* __restrict__ p,
             const TC* __restrict__ Hp, const TC* __restrict__ D, TC c, size_t n3,
             RedArgs ra, double rtol2, int max_iter) {
@@ -590,10 +632,10 @@ k_cg_update(TC* __restrict__ x, TC* __restrict__ r, const TC* __restrict__ p,
       xv.v[j] = xn;
       const TC ri = rv.v[j] - alpha * hv.v[j];
       rv.v[j] = ri;
-      const TC zi = JAC ? jacobi(ri, dv.v[j], c) : ri;
+      const TC zi = JAC ? jprec(ri, dv.v[j], c) : ri;
       a0.add(ri * zi);
       a1.add(ri * ri);
-      a2.max(xn < (TC)0 ? -xn : xn);
+      a2.maxabs(xn);
     }
     st4(x + i, xv);
     st4(r + i, rv);
@@ -638,9 +680,10 @@ k_newton_update(const T* __restrict__ s, const T* __restrict__ y, const T* __res
                 T* __restrict__ y2, T* __restrict__ g2, TC* __restrict__ D2,
                 TC* __restrict__ r2, size_t n3, RedArgs ra) {
   using Acc = typename AccOf<T>::type;
-  Acc acc[6];
+  constexpr int NS = sizeof(TC) == 8 ? 5 : 6;   // k_precond takes the last sum (FP64 CG)
+  Acc acc[NS];
 #pragma unroll
-  for (int j = 0; j < 6; ++j) acc[j].init(false);
+  for (int j = 0; j < NS; ++j) acc[j].init(false);
   const double tau = tau_dev ? *tau_dev : tau_arg;
   const T tt = (T)tau, nb = (T)nbar, m = (T)mu;
   const TC cc = (TC)c;
@@ -662,7 +705,7 @@ k_newton_update(const T* __restrict__ s, const T* __restrict__ y, const T* __res
       const TC sinv_xi = b_j - rv.v[j] - dv.v[j] * xv.v[j];
       const T yn = yv.v[j] + tt * (T)sinv_xi;
       const T sn = sv.v[j] + tt * (T)xv.v[j];
-      const T d = nb * (T)wv.v[j] * exp(sn);
+      const T d = nb * (T)wv.v[j] * expt(sn);
       const T ni = (T)nv.v[j];
       const T gn = yn + d - ni;
       so.v[j] = sn;
@@ -676,8 +719,10 @@ k_newton_update(const T* __restrict__ s, const T* __restrict__ y, const T* __res
       const TC nc = (TC)nv.v[j], sc = (TC)sn;
       acc[3].add((T)(nc * sc));
       acc[4].add((T)(nc * (sc < (TC)0 ? -sc : sc)));
-      const TC gc = (TC)gn;
-      acc[5].add((T)(jac ? gc * jacobi(gc, (TC)d, cc) : gc * gc));
+      if constexpr (NS > 5) {
+        const TC gc = (TC)gn;
+        acc[5].add((T)(jac ? gc * jacobi(gc, (TC)d, cc) : gc * gc));
+      }
     }
     st4(s2 + i, so);
     st4(y2 + i, yo);
@@ -685,7 +730,7 @@ k_newton_update(const T* __restrict__ s, const T* __restrict__ y, const T* __res
     st4(D2 + i, dout);
     st4(r2 + i, rout);
   }
-  block_reduce_finish_acc<6, 0u>(acc, ra, FinGrad{});
+  block_reduce_finish_acc<NS, 0u>(acc, ra, FinGrad<NS>{});
 }
 
 // D = nbar w e^s (Sec. 3.1.2), from an FP64 s.
@@ -695,7 +740,7 @@ k_diag(const double* __restrict__ s, const double* __restrict__ w, double nbar,
        TC* __restrict__ D, size_t n3) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n3;
        i += (size_t)gridDim.x * blockDim.x)
-    D[i] = (TC)(nbar * (w ? w[i] : 1.0) * exp(s[i]));
+    D[i] = (TC)(nbar * (w ? w[i] : 1.0) * exp64(s[i]));
 }
 
 // Lambert W of x = e^L from L = ln x (x up to e^300 and beyond), in FP32:
@@ -814,7 +859,7 @@ k_newton_update_g(const T* __restrict__ s, const T* __restrict__ y, const T* __r
     st4(D2 + i, dout);
     st4(r2 + i, rout);
   }
-  block_reduce_finish_acc<6, 0u>(acc, ra, FinGrad{});
+  block_reduce_finish_acc<6, 0u>(acc, ra, FinGrad<6>{});
 }
 
 // Fraction to the boundary of the Gaussian-prior model: the largest

@@ -535,25 +535,21 @@ kx_xi(const fxc* __restrict__ A, FxExps ex, Epi epi, Fin fin, RedArgs ra,
     }
   }
   __syncthreads();
-  // doubles by integer operations; exponents outside their range (NaN tiles,
-  // all-zero grids, values near the ends of the double range) by ldexp
   const bool plain = E > -900 && E < 900;
-  auto value = [&](fx q) -> double {
-    if (plain) return fx_to_double(q, E);
-    if (E >= kFxNaN / 2) return __longlong_as_double(0x7ff8000000000000ll);
-    return q.v == 0 ? 0.0 : ldexp((double)q.v, max(E, -4000));
-  };
+  auto value = [&](long long q) { return plain ? fx_to_double(fx{q}, E) : fx_to_double_far(q, E); };
   typename Epi::Acc acc[Epi::NV > 0 ? Epi::NV : 1];
 #pragma unroll
   for (int j = 0; j < Epi::NV; ++j) acc[j].init((Epi::MAXMASK >> j) & 1u);
   constexpr int Q = N / 4, TOT = Gm::RY * Q;
+// one step at a time: unrolled by 2 or 4, with e^s in the loop, it outgrows
+// the instruction cache (public H v at 256^3: 254, 260 and 276 us)
 #pragma unroll 1
   for (int e = threadIdx.x; e < TOT; e += kThreads) {
     const int row = e / Q, x = 4 * (e % Q);
     const longlong2 a = reinterpret_cast<const longlong2*>(&R[row * Gm::SR + x])[0];
     const longlong2 b = reinterpret_cast<const longlong2*>(&R[row * Gm::SR + x])[1];
     epi.vec4(row0 + (size_t)row * N + x,
-             V4<double>{{value(fx{a.x}), value(fx{a.y}), value(fx{b.x}), value(fx{b.y})}}, acc);
+             V4<double>{{value(a.x), value(a.y), value(b.x), value(b.y)}}, acc);
   }
   if constexpr (Epi::NV > 0) block_reduce_finish_acc<Epi::NV, Epi::MAXMASK>(acc, ra, fin);
 }

@@ -62,6 +62,7 @@ int run_cg(plc_ctx* c, TC* x, TC* r, TC* p, TC* Hp, const TC* D, bool jac, doubl
            int max_cg, int chunk, int first) {
   int launched = 0;
   int k = std::max(1, std::min(first, chunk));
+  precond<TC>(c, D, r, jac);
   read_scalars(c);
   while (!c->sc_host->done && launched < max_cg) {
     k = std::min(k, max_cg - launched);

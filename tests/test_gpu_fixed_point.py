@@ -97,3 +97,30 @@ def test_zero_and_non_finite_fields(plc, n):
         assert not bool(torch.isfinite(c.prior_apply(x)).any())
     x.normal_()
     assert bool(torch.isfinite(c.prior_apply(x)).all())   # nothing of it stays behind
+
+
+def test_exponential_to_the_last_place(plc):
+    # a constant v lies in the DC mode, whose eigenvalue is infinite, so
+    # H v = nbar e^s v exactly.  Within |s| < 32 the integer exponential is one
+    # rounding (half an ulp) of a value within 2^-56.6 (0.09 ulp); outside the
+    # library function allows one ulp.
+    n = 32
+    c = _context(plc, n)
+    rng = np.random.default_rng(3)
+    s = np.concatenate([rng.uniform(-33, 33, n ** 3 // 2), 3.0 * rng.standard_normal(n ** 3 // 2)])
+    edge = [0.0, -0.0, 1e-300, -5e-324, 2.0 ** -60, -2.0 ** -53, 31.999999999999996, -31.999999999999996,
+            32.0, -32.0, 40.0, 709.7, 710.0, -700.0, -746.0, np.log(2.0), np.log(2.0) / 128,
+            -np.log(2.0) / 128, float("inf"), -float("inf"), float("nan")]
+    s[:len(edge)] = edge
+    one = torch.ones((n, n, n), dtype=torch.float64, device="cuda")
+    y = host(c.hessvec(dev(s.reshape(n, n, n), torch.float64), None, 1.0, one)).ravel()
+    with np.errstate(over="ignore", under="ignore"):
+        ref = np.exp(s.astype(np.longdouble))
+        want = ref.astype(np.float64)
+    assert np.array_equal(np.isnan(y), np.isnan(want))
+    inf = np.isinf(want)
+    assert np.array_equal(y[inf], want[inf])
+    ok = np.isfinite(want)
+    ulps = np.abs(y[ok].astype(np.longdouble) - ref[ok]) / np.spacing(want[ok])
+    assert float(np.max(ulps[np.abs(s[ok]) < 32])) <= 0.6
+    assert float(np.max(ulps)) <= 1.0
