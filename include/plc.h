@@ -273,7 +273,7 @@ plc_status plc_compare(plc_ctx* ctx, const double* a, const double* b, double* r
  * 5 and 10 Mpc/h before the matter statistics): y = x convolved with a
  * normalised Gaussian of radius `radius` (Mpc/h, >= 0), i.e. every Fourier
  * mode multiplied by exp(-|k|^2 radius^2 / 2), |k| as for the prior.  x, y:
- * double fields (may alias).  Transforms in float-float (about 48 bits) for
+ * double fields (may alias).  Transforms in 64-bit block fixed point for
  * lengths with a four-step schedule, FP64 otherwise; uses the solver work
  * fields as scratch.  Needs no prior.  Synchronises the stream. */
 plc_status plc_smooth(plc_ctx* ctx, const double* x, double* y, double radius);

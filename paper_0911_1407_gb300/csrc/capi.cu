@@ -88,7 +88,7 @@ template <typename T> void dalloc(T** p, size_t bytes) {
 void release(plc_ctx* c) {
   plc::graph_release(c);
   plc::profile_release(c);
-  void* ptrs[] = {c->specA, c->specB, c->tw64, c->tw32, c->twfx, c->fxexp, c->twff, c->expff, c->M64, c->M32,
+  void* ptrs[] = {c->specA, c->specB, c->tw64, c->tw32, c->twfx, c->fxexp, c->expff, c->M64, c->M32,
                   c->lk, c->lP, c->sc, c->partials, c->Mb64, c->Mb32, c->lkb, c->lbb, c->hist};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -228,7 +228,6 @@ plc_status plc_create(plc_ctx** out, int n, double box, int precision, void* str
     dalloc(&c->tw32, sizeof(float2) * n);
     dalloc(&c->twfx, sizeof(plc::fxw) * n);
     dalloc(&c->fxexp, sizeof(int) * plc::fx_exps_ints(n));
-    dalloc(&c->twff, sizeof(float4) * n);
     dalloc(&c->expff, sizeof(float2) * 64);
     dalloc(&c->sc, sizeof(plc::DevScalars));
     plc::check(cudaMallocHost(reinterpret_cast<void**>(&c->sc_host), sizeof(plc::DevScalars)),
@@ -240,7 +239,6 @@ plc_status plc_create(plc_ctx** out, int n, double box, int precision, void* str
     std::vector<double2> t64(n);
     std::vector<float2> t32(n);
     std::vector<plc::fxw> tfx(n);
-    std::vector<float4> tff(n);   // float-float: (re hi, re lo, im hi, im lo)
     for (int m = 0; m < n; ++m) {
       const double ang = 2.0 * M_PI * (double)m / (double)n;
       t64[m] = make_double2(std::cos(ang), -std::sin(ang));
@@ -250,13 +248,10 @@ plc_status plc_create(plc_ctx** out, int n, double box, int precision, void* str
       tfx[m] = plc::fxw{plc::fx_split(std::llrint(std::cos(al) * one)),
                         plc::fx_split(std::llrint(-std::sin(al) * one))};
       t32[m] = make_float2((float)t64[m].x, (float)t64[m].y);
-      tff[m] = make_float4(t32[m].x, (float)(t64[m].x - (double)t32[m].x), t32[m].y,
-                           (float)(t64[m].y - (double)t32[m].y));
     }
     plc::check(cudaMemcpyAsync(c->tw64, t64.data(), sizeof(double2) * n, cudaMemcpyHostToDevice, c->stream), "copy twiddles");
     plc::check(cudaMemcpyAsync(c->tw32, t32.data(), sizeof(float2) * n, cudaMemcpyHostToDevice, c->stream), "copy twiddles");
     plc::check(cudaMemcpyAsync(c->twfx, tfx.data(), sizeof(plc::fxw) * n, cudaMemcpyHostToDevice, c->stream), "copy twiddles");
-    plc::check(cudaMemcpyAsync(c->twff, tff.data(), sizeof(float4) * n, cudaMemcpyHostToDevice, c->stream), "copy twiddles");
     // 2^(j/64), j < 64, in float-float (the table of the float-float exp)
     std::vector<float2> e2(64);
     for (int j = 0; j < 64; ++j) {

@@ -80,6 +80,7 @@ struct DevScalars {
 template <typename C> __device__ __forceinline__ C cmk(decltype(C::x) a, decltype(C::x) b) {
   C r; r.x = a; r.y = b; return r;
 }
+__device__ __forceinline__ float halve(float a) { return 0.5f * a; }   // exact
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return cmk<C>(a.x + b.x, a.y + b.y); }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { return cmk<C>(a.x - b.x, a.y - b.y); }
 template <typename C> __device__ __forceinline__ C cmul(C a, C b) {

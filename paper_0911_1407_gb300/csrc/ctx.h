@@ -21,7 +21,8 @@ enum Site {
   // pipelines of the Newton gradient (and line-search trials)
   S_GXF64, S_GYF64, S_GZ64, S_GYI64, S_GXI64,
   S_GXF32, S_GYF32, S_GZ32, S_GYI32, S_GXI32,
-  // the FP64 gradient of the mixed solve in float-float transforms
+  // the FP64 gradient of the mixed solve and the smoothing, in fixed-point
+  // transforms (the names' "ff": the gradient's float-float epilogue)
   S_GXFF, S_GYFF, S_GZFF, S_GYIFF, S_GXIFF,
   S_CG_INIT, S_CG_UPDATE64, S_CG_UPDATE32, S_NEWTON_UPDATE64, S_NEWTON_UPDATE32,
   S_DIAG, S_CONVERT, S_SETUP, S_BOUNDARY,
@@ -72,7 +73,6 @@ struct plc_ctx {
   float2* tw32 = nullptr;
   void* twfx = nullptr;        // fixed-point twiddles (fxw, fx.cuh)
   int* fxexp = nullptr;        // tile exponents of the fixed-point spectra (FxExps)
-  void* twff = nullptr;        // float-float twiddles (ffc, ff.cuh)
   void* expff = nullptr;       // 2^(j/64), j < 64, float-float (exp_ff)
 
   // Prior: inverse eigenvalue per |m|^2, its FP32 copy, ln-tables.
@@ -149,7 +149,7 @@ template <typename T, typename TS, typename TC>
 void grad_newton(plc_ctx* c, const TS* s, const double* w, const int32_t* N, double nbar, T* y,
                  T* g, TC* D, TC* r, bool jac);
 // Newton trial point s + tau xi without an FFT (see k_newton_update).
-// The sums of the FP64 gradient of the mixed solve at s (float-float
+// The sums of the FP64 gradient of the mixed solve at s (fixed-point
 // transforms, no field stored) into sc->red; false when the length has no
 // four-step schedule (nothing launched).
 bool grad_sums_ff(plc_ctx* c, const double* s, const double* w, const int32_t* N, double nbar,

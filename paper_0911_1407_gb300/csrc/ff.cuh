@@ -30,11 +30,6 @@ struct __align__(8) ff {
       : hi((float)d), lo((float)(d - (double)(float)d)) {}
 };
 
-struct __align__(16) ffc {
-  ff x, y;
-};
-template <> struct CplxOf<ff> { using type = ffc; };
-
 __device__ __forceinline__ ff operator+(ff a, ff b) {
   const float s = a.hi + b.hi;
   const float bb = s - a.hi;
@@ -52,15 +47,6 @@ __device__ __forceinline__ ff operator*(ff a, ff b) {
   const float h = p + e;
   return ff(h, e - (h - p));
 }
-// sign factors of the small DFTs (+-1)
-__device__ __forceinline__ ff operator*(int s, ff a) {
-  return s == 1 ? a : (s == -1 ? -a : ff((double)s) * a);
-}
-
-// exact halving
-__device__ __forceinline__ float halve(float a) { return 0.5f * a; }
-__device__ __forceinline__ ff halve(ff a) { return ff(0.5f * a.hi, 0.5f * a.lo); }
-
 __device__ __forceinline__ double to_double(ff a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ double to_double(float a) { return (double)a; }
 

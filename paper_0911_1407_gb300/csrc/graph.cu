@@ -449,7 +449,7 @@ void capture_solve(plc_ctx* c, cudaGraph_t top, const std::vector<cudaStream_t>&
   // a conditional node for the graph to instantiate)
   const int first = o.start == 0 ? 0 : (o.g0_norm > 0.0 ? 2 : (o.start == 2 ? 3 : 1));
   if (first == 1) mk(&h_first);
-  // the switch's sums-only check: mixed solves of lengths with float-float
+  // the switch's sums-only check: mixed solves of lengths with fixed-point
   // transforms (a four-step schedule)
   bool has_check = false;
   if constexpr (kMixed) {

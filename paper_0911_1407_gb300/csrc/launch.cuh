@@ -38,27 +38,21 @@ template <auto Kernel> inline void set_smem4(size_t bytes) {
   check(once, "cudaFuncSetAttribute");
 }
 
-// The passes with register four-step line transforms (passes4.cuh) in
-// transform arithmetic T: float (FP32 twiddles and multipliers) or ff
-// (float-float, from the FP64 tables).
+// The passes with register four-step line transforms (passes4.cuh) in FP32.
 template <typename T, int N1, int N2, typename Pro, typename Epi, typename Fin>
 void run_pipeline4(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* done, int s0,
-                   const void* m_override = nullptr) {
+                   const T* m_override = nullptr) {
   using Gm = Geo4<T, N1, N2>;
   using C = cpx<T>;
-  constexpr bool kFF = std::is_same<T, ff>::value;
-  using TM = typename std::conditional<kFF, double, float>::type;
   constexpr int n = Gm::N, h = n / 2 + 1;
   C* A = static_cast<C*>(c->specA);
   C* B = static_cast<C*>(c->specB);
-  const C* tw = kFF ? static_cast<const C*>(c->twff) : reinterpret_cast<const C*>(c->tw32);
-  const TM* M = m_override ? static_cast<const TM*>(m_override)
-                           : kFF ? reinterpret_cast<const TM*>(c->M64)
-                                 : reinterpret_cast<const TM*>(c->M32);
+  const C* tw = twiddles<T>(c);
+  const T* M = m_override ? m_override : multiplier<T>(c);
   const dim3 gx(n / Gm::RY, n), gy(n / Gm::L, h);
   set_smem4<k4_xf<T, N1, N2, Pro>>(Gm::smem_x);
   set_smem4<k4_yf<T, N1, N2>>(Gm::smem_y);
-  set_smem4<k4_z<T, N1, N2, TM>>(Gm::smem_z);
+  set_smem4<k4_z<T, N1, N2>>(Gm::smem_z);
   set_smem4<k4_yi<T, N1, N2>>(Gm::smem_y);
   set_smem4<k4_xi<T, N1, N2, Epi, Fin>>(Gm::smem_x);
   {
@@ -71,7 +65,7 @@ void run_pipeline4(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int
   }
   {
     LaunchScope ls(c, Site(s0 + 2));
-    k4_z<T, N1, N2, TM><<<gy, kThreads, Gm::smem_z, c->stream>>>(B, M, zero_dc, tw, done);
+    k4_z<T, N1, N2><<<gy, kThreads, Gm::smem_z, c->stream>>>(B, M, zero_dc, tw, done);
   }
   {
     LaunchScope ls(c, Site(s0 + 3));
@@ -89,7 +83,7 @@ void run_pipeline4(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int
 // ctx.h); false when the plan has none (Stockham stages).
 template <typename T, typename Pro, typename Epi, typename Fin>
 bool run_four_step(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* done, int s0,
-                   const void* m_override = nullptr) {
+                   const T* m_override = nullptr) {
   switch (c->plan.f1 * 64 + c->plan.f2) {
     case 16 * 64 + 16: run_pipeline4<T, 16, 16>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
     case 16 * 64 + 12: run_pipeline4<T, 16, 12>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
@@ -235,11 +229,13 @@ template <typename T, typename TS, typename TC>
 void grad_newton(plc_ctx* c, const TS* s, const double* w, const int32_t* N, double nbar, T* y,
                  T* g, TC* D, TC* r, bool jac) {
   if constexpr (std::is_same<T, double>::value && std::is_same<TC, float>::value) {
-    // the FP64 gradient of the mixed solve: float-float transforms and
-    // epilogue where the length has a four-step schedule
+    // the FP64 gradient of the mixed solve: fixed-point transforms and a
+    // float-float epilogue where the length has a four-step schedule
     const EpiGradFF<true> epi{s, w, N, ff(nbar), ff(c->mu), y, g, D, r, (float)c->jac_c,
                               jac ? 1 : 0, static_cast<const ff*>(c->expff)};
-    if (run_four_step<ff>(c, ProShiftFF{s, ff(c->mu)}, epi, FinGrad<6>{}, 0, nullptr, S_GXFF)) return;
+    if (run_fixed(c, ProShift<double, double>{s, c->mu}, epi, FinGrad<6>{}, 0, nullptr, S_GXFF,
+                  nullptr))
+      return;
   }
   constexpr int NS = sizeof(TC) == 8 ? 5 : 6;
   run_pipeline<T>(c, ProShift<T, TS>{s, c->mu},
@@ -249,15 +245,16 @@ void grad_newton(plc_ctx* c, const TS* s, const double* w, const int32_t* N, dou
 }
 
 // The sums of the FP64 gradient of the mixed solve at an FP64 s (the
-// float-float pipeline with nothing stored: -ln P, ||g||^2 and the scale of
-// the rounding test into sc->red, FinGrad), for a stopping test that may end
-// the solve before the gradient's fields are needed.  False (nothing run)
+// same pipeline with nothing stored: the sums of -ln P and ||g||^2 into
+// sc->red, FinGrad), for a stopping test that may end the solve before the
+// gradient's fields are needed.  False (nothing run)
 // when the length has no four-step schedule.
 inline bool grad_sums_ff_impl(plc_ctx* c, const double* s, const double* w, const int32_t* N,
                               double nbar, bool jac) {
   const EpiGradFF<false> epi{s, w, N, ff(nbar), ff(c->mu), nullptr, nullptr, nullptr, nullptr,
                              (float)c->jac_c, jac ? 1 : 0, static_cast<const ff*>(c->expff)};
-  return run_four_step<ff>(c, ProShiftFF{s, ff(c->mu)}, epi, FinGrad<6>{}, 0, nullptr, S_GXFF);
+  return run_fixed(c, ProShift<double, double>{s, c->mu}, epi, FinGrad<3>{}, 0, nullptr, S_GXFF,
+                   nullptr);
 }
 
 template <typename T, typename TS, typename TC>

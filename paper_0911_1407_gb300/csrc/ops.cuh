@@ -6,7 +6,7 @@
 // finalizers run once on the grid totals.  Element-wise kernels cover the CG
 // recurrences and set-up work.  Reductions accumulate per thread in the
 // field's own precision made compensated (Kahan pairs for FP32 fields,
-// float-float for the float-float transforms, plain FP64 for FP64 fields),
+// float-float for the mixed solve's FP64 gradient, plain FP64 for FP64 fields),
 // merge across lanes and warps in that arithmetic, and go to FP64 once per
 // block; the block totals are summed in FP64 in block order.
 #pragma once
@@ -121,30 +121,32 @@ template <typename T, bool JAC> struct ProCgDir {
   }
 };
 
-// s - mu from an FP64 s, in float-float for float-float transforms: s split
-// into float-float by its bit fields, mu given as a float-float (error a few
-// 2^-48 of max(|s|, |mu|)).
-struct ProShiftFF {
-  const double* s;
-  ff mu;
-  __device__ void prepare() {}
-  __device__ void prefetch(size_t i, unsigned cnt) const { prefetch_l2(s + i, cnt * sizeof(double)); }
-  __device__ V4<ff> vec4(size_t i) const {
-    const V4<double> a = ld4(s + i);
-    return V4<ff>{{ff_split(a.v[0]) - mu, ff_split(a.v[1]) - mu, ff_split(a.v[2]) - mu,
-                   ff_split(a.v[3]) - mu}};
-  }
-};
-
 // ------------------------------- epilogues --------------------------------
-// The gradient epilogue of EpiGrad for float-float transforms (the FP64
-// gradient of the mixed solve), kept in float-float: y (from the transform),
-// s (FP64 in memory, split by its bit fields), D = nbar w e^s (exp_ff),
-// g = y + D - N and the six sums of EpiGrad are float-float; y and g are
-// stored in FP64, D and r = -g in FP32.  With STORE false nothing is stored
-// (the sums alone, for a stopping test that may end the solve).
+// q 2^E as a float-float: the three parts of q (22, 24 and 16 bits) as floats,
+// the upper two added exactly and the third to their rounding error.
+__device__ __forceinline__ ff fx_to_ff(fx q, int E) {
+  if (E <= -110 || E >= 50) return ff(fx_to_double_far(q.v, E));   // uniform, rare
+  auto p2 = [](int e) { return __uint_as_float((unsigned)(127 + e) << 23); };
+  const float a = (float)((int)(q.v >> 32) >> 8) * p2(E + 40);
+  const float b = (float)((unsigned)(q.v >> 16) & 0xffffffu) * p2(E + 16);
+  const float c = (float)((unsigned)q.v & 0xffffu) * p2(E);
+  const float h = a + b;                     // |a| >= b or a = 0 (Fast2Sum)
+  const float l = (b - (h - a)) + c;
+  const float s = h + l;
+  return ff(s, l - (s - h));
+}
+
+// The gradient epilogue of EpiGrad for the FP64 gradient of the mixed solve,
+// kept in float-float on the FP32 pipes (an FP64 pipe that issues two
+// operations per SM and clock would bound it): y straight from the transform's
+// integers (kRaw), s (FP64 in memory, split by its bit fields), D = nbar w e^s
+// (exp_ff), g = y + D - N and the six sums of EpiGrad are float-float; y and g
+// are stored in FP64, D and r = -g in FP32.  With STORE false nothing is
+// stored and only the sums of -ln P and ||g||^2 are taken (for a stopping test
+// that may end the solve).
 template <bool STORE = true> struct EpiGradFF {
-  static constexpr int NV = 6;
+  static constexpr int NV = STORE ? 6 : 3;
+  static constexpr bool kRaw = true;
   static constexpr unsigned MAXMASK = 0;
   using Acc = AccFF;
   const double* s;
@@ -163,7 +165,7 @@ template <bool STORE = true> struct EpiGradFF {
     prefetch_l2(N + i, cnt * sizeof(int32_t));
     if (w) prefetch_l2(w + i, cnt * sizeof(double));
   }
-  __device__ void vec4(size_t i, const V4<ff>& y, Acc* acc) const {
+  __device__ void vec4(size_t i, const V4<fx>& q, int E, Acc* acc) const {
     const V4<double> sv = ld4(s + i);
     const V4<int32_t> nv = ld4(N + i);
     V4<double> wv{{1.0, 1.0, 1.0, 1.0}};
@@ -177,17 +179,18 @@ template <bool STORE = true> struct EpiGradFF {
       ff d = nb * exp_ff(st, exptab);
       if (w) d = d * ff_split(wv.v[j]);
       const ff ni((float)nv.v[j], 0.f);    // counts below 2^24 are exact
-      const ff gi = (y.v[j] + d) - ni;
+      const ff y = fx_to_ff(q.v[j], E);
+      const ff gi = (y + d) - ni;
       const ff ns = ni * st;
-      acc[0].add((st - m) * y.v[j]);
+      acc[0].add((st - m) * y);
       acc[1].add(d - ns);
       acc[2].add(gi * gi);
-      acc[3].add(ns);
-      acc[4].add(ni * ff_abs(st));
-      const float gc = gi.hi + gi.lo, dc = d.hi + d.lo;
-      acc[5].add(ff(jac ? gc * jacobi(gc, dc, c) : gc * gc, 0.f));
       if constexpr (STORE) {
-        yo.v[j] = to_double(y.v[j]);
+        acc[3].add(ns);
+        acc[4].add(ni * ff_abs(st));
+        const float gc = gi.hi + gi.lo, dc = d.hi + d.lo;
+        acc[5].add(ff(jac ? gc * jacobi(gc, dc, c) : gc * gc, 0.f));
+        yo.v[j] = to_double(y);
         go.v[j] = to_double(gi);
         dv.v[j] = dc;
         rv.v[j] = -gc;
@@ -199,20 +202,6 @@ template <bool STORE = true> struct EpiGradFF {
       if (D) st4(D + i, dv);
       if (r) st4(r + i, rv);
     }
-  }
-};
-
-// An FP64 epilogue behind float-float transforms: y = hi + lo in FP64.
-template <typename Epi> struct EpiFF {
-  static constexpr int NV = Epi::NV;
-  static constexpr unsigned MAXMASK = Epi::MAXMASK;
-  using Acc = typename Epi::Acc;
-  Epi epi;
-  __device__ void prefetch(size_t i, unsigned cnt) const { epi.prefetch(i, cnt); }
-  __device__ void vec4(size_t i, const V4<ff>& y, Acc* acc) const {
-    const V4<double> yd{{to_double(y.v[0]), to_double(y.v[1]), to_double(y.v[2]),
-                         to_double(y.v[3])}};
-    epi.vec4(i, yd, acc);
   }
 };
 
@@ -475,7 +464,7 @@ template <int NV> struct FinStore {
 // After a gradient: store the sums and start CG on H xi = -g from xi = 0
 // (r = -g was written by the epilogue).  The CG tolerance and iteration cap
 // are arguments of the CG update.  NS = 5: r^T M^-1 r is ||r||^2 (M = I) until
-// k_precond sets it.
+// k_precond sets it; NS = 3: a stopping test, no CG follows.
 template <int NS> struct FinGrad {
   __device__ void operator()(const double* t, DevScalars* sc) const {
 #pragma unroll

@@ -33,11 +33,10 @@
 // keep their 16-byte vector accesses.
 //
 // T is the arithmetic of the transforms: float (the FP32 operators and the
-// FP32 phase of the solve) or ff, float-float on the FP32 pipes (ff.cuh),
-// for the FP64 gradient of the mixed solve.
+// FP32 phase of the solve).  FP64 fields take the fixed-point form of these
+// passes (passesx.cuh), which shares the geometry.
 #pragma once
 
-#include "ff.cuh"
 #include "ops.cuh"
 #include "passes.cuh"
 
@@ -157,11 +156,6 @@ k4_yf(const cpx<T>* __restrict__ A, cpx<T>* __restrict__ B, const cpx<T>* __rest
   }
 }
 
-// A multiplier of the z pass in the transform arithmetic (float, or
-// float-float split from the FP64 table without the FP64 pipe).
-__device__ __forceinline__ float as_mult(float m, float) { return m; }
-__device__ __forceinline__ ff as_mult(double m, ff) { return ff_split(m); }
-
 // Resident blocks per SM asked of the compiler for the z pass.  FP32 at
 // 16 x 16: three blocks (up to 85 registers, it takes 69) ran the pass at
 // 256^3 in 32.8 us against 36.9 us at four blocks of 59 registers on
@@ -180,9 +174,9 @@ template <> struct ZMinBlocks<float, 16, 16> { static constexpr int value = 3; }
 // one task of each phase (L N1 = L N2 = kThreads) the guards and the task
 // loop are compiled out.
 // ---------------------------------------------------------------------------
-template <typename T, int N1, int N2, typename TM>
+template <typename T, int N1, int N2>
 __global__ void __launch_bounds__(kThreads, ZMinBlocks<T, N1, N2>::value)
-k4_z(cpx<T>* __restrict__ B, const TM* __restrict__ M, int zero_dc,
+k4_z(cpx<T>* __restrict__ B, const T* __restrict__ M, int zero_dc,
      const cpx<T>* __restrict__ twg, const int* __restrict__ done) {
   PLC_PASS4_PROLOGUE(C* X = tw2 + N; T* Ms = reinterpret_cast<T*>(X + Gm::L * Gm::S));
   // planes in decreasing kx: the y-forward pass before it writes them in
@@ -209,8 +203,7 @@ k4_z(cpx<T>* __restrict__ B, const TM* __restrict__ M, int zero_dc,
     const int c = i / HM, mz = i - c * HM;
     const int ky = ky0 + c, my = min(ky, N - ky);
     const int m2 = kx * kx + my * my + mz * mz;
-    mv[j] = (i >= Gm::L * HM || (zero_dc && m2 == 0)) ? as_mult(TM(0), T())
-                                                       : as_mult(__ldg(M + m2), T());
+    mv[j] = (i >= Gm::L * HM || (zero_dc && m2 == 0)) ? T(0) : __ldg(M + m2);
   }
 #pragma unroll
   for (int j = 0; j < MI; ++j) {
@@ -299,7 +292,6 @@ template <int N1> __device__ __forceinline__ int pair_k1(int g, int member) {
 }
 
 __device__ __forceinline__ float shfl_xor16(float a) { return __shfl_xor_sync(0xffffffffu, a, 16); }
-__device__ __forceinline__ ff shfl_xor16(ff a) { return ff(shfl_xor16(a.hi), shfl_xor16(a.lo)); }
 template <typename C> __device__ __forceinline__ C shfl_xor16(C a) {
   return cmk<C>(shfl_xor16(a.x), shfl_xor16(a.y));
 }
@@ -308,27 +300,9 @@ template <typename C> __device__ __forceinline__ C shfl_xor16(C a) {
 __device__ __forceinline__ void st_row4(float* p, const V4<float>& u) {
   *reinterpret_cast<float4*>(p) = make_float4(u.v[0], u.v[1], u.v[2], u.v[3]);
 }
-__device__ __forceinline__ void st_row4(ff* p, const V4<ff>& u) {
-  reinterpret_cast<float4*>(p)[0] = make_float4(u.v[0].hi, u.v[0].lo, u.v[1].hi, u.v[1].lo);
-  reinterpret_cast<float4*>(p)[1] = make_float4(u.v[2].hi, u.v[2].lo, u.v[3].hi, u.v[3].lo);
-}
 __device__ __forceinline__ V4<float> ld_row4(const float* p) {
   const float4 q = *reinterpret_cast<const float4*>(p);
   return V4<float>{{q.x, q.y, q.z, q.w}};
-}
-__device__ __forceinline__ V4<ff> ld_row4(const ff* p) {
-  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
-  return V4<ff>{{ff(a.x, a.y), ff(a.z, a.w), ff(b.x, b.y), ff(b.z, b.w)}};
-}
-
-// A pair of adjacent complex values (the spectra of the two packed rows).
-__device__ __forceinline__ void ld_pair(const ffc* p, ffc& a, ffc& b) {
-  a = p[0];
-  b = p[1];
-}
-__device__ __forceinline__ void st_pair(ffc* p, ffc a, ffc b) {
-  p[0] = a;
-  p[1] = b;
 }
 
 // ---------------------------------------------------------------------------
@@ -337,16 +311,6 @@ __device__ __forceinline__ void st_pair(ffc* p, ffc a, ffc b) {
 // Z = FFT(row_2c + i row_2c+1): X_a[k] = (Z[k] + conj Z[N-k]) / 2 and
 // X_b[k] = (Z[k] - conj Z[N-k]) / 2i, stored as a pair at A[z][k][y0+2c].
 // ---------------------------------------------------------------------------
-// Resident blocks per SM the x-forward pass asks the compiler for: 1 (no
-// register cap) except for the float-float prologue of the refresh gradient,
-// which at 3 blocks (80 registers, shared memory allows 3) measured 152 us
-// against 164 at 2 (89 registers) for 256^3.
-template <typename Pro> struct XfMinBlocks {
-  static constexpr int value = 1;
-};
-template <> struct XfMinBlocks<ProShiftFF> {
-  static constexpr int value = 3;
-};
 // Prologue steps (four x each) a thread keeps in flight: eight, or
 // Pro::kBatch where the prologue sets one.
 template <typename Pro, typename = void> struct XfBatch {
@@ -357,7 +321,7 @@ template <typename Pro> struct XfBatch<Pro, decltype((void)Pro::kBatch)> {
 };
 
 template <typename T, int N1, int N2, typename Pro>
-__global__ void __launch_bounds__(kThreads, XfMinBlocks<Pro>::value)
+__global__ void __launch_bounds__(kThreads, 1)
 k4_xf(Pro pro, cpx<T>* __restrict__ A, const cpx<T>* __restrict__ twg,
       const int* __restrict__ done) {
   PLC_PASS4_SETUP(T* R = reinterpret_cast<T*>(tw2 + N); C* X = tw2 + N);
@@ -455,19 +419,8 @@ template <typename Epi> struct EpiUnroll<Epi, decltype((void)Epi::kUnroll)> {
 // (projection onto real fields).  The epilogue sees y = (S^-1 x)_i per cell
 // and accumulates Epi::NV sums; Fin runs once on the grid totals.
 // ---------------------------------------------------------------------------
-// Resident blocks per SM the x-inverse pass asks the compiler for: 1 (no
-// register cap) except for the float-float gradient epilogue, which at 3
-// blocks (80 registers, 32 bytes of spill; shared memory allows 3) measured
-// 471 us against 598 at 2 blocks (128 registers) for 256^3.
-template <typename Epi> struct XiMinBlocks {
-  static constexpr int value = 1;
-};
-template <bool STORE> struct XiMinBlocks<EpiGradFF<STORE>> {
-  static constexpr int value = 3;
-};
-
 template <typename T, int N1, int N2, typename Epi, typename Fin>
-__global__ void __launch_bounds__(kThreads, XiMinBlocks<Epi>::value)
+__global__ void __launch_bounds__(kThreads, 1)
 k4_xi(const cpx<T>* __restrict__ A, Epi epi, Fin fin, RedArgs ra,
       const cpx<T>* __restrict__ twg, const int* __restrict__ done) {
   PLC_PASS4_PROLOGUE(T* R = reinterpret_cast<T*>(tw2 + N); C* X = tw2 + N);

@@ -454,6 +454,14 @@ kx_yi(const fxc* __restrict__ B, fxc* __restrict__ A, FxExps ex, const fxw* __re
 // form for N - k have L1 norms of at most |X_a| + |X_b| each, so a line's is
 // bounded by twice the sum over k <= n/2.
 // ---------------------------------------------------------------------------
+// Epilogues that take the transform's integers and exponent (Epi::kRaw).
+template <typename Epi, typename = void> struct EpiRaw {
+  static constexpr bool value = false;
+};
+template <typename Epi> struct EpiRaw<Epi, decltype((void)Epi::kRaw)> {
+  static constexpr bool value = Epi::kRaw;
+};
+
 template <int N1, int N2, typename Epi, typename Fin>
 __global__ void __launch_bounds__(kThreads, kFxBlocks)
 kx_xi(const fxc* __restrict__ A, FxExps ex, Epi epi, Fin fin, RedArgs ra,
@@ -548,7 +556,10 @@ kx_xi(const fxc* __restrict__ A, FxExps ex, Epi epi, Fin fin, RedArgs ra,
     const int row = e / Q, x = 4 * (e % Q);
     const longlong2 a = reinterpret_cast<const longlong2*>(&R[row * Gm::SR + x])[0];
     const longlong2 b = reinterpret_cast<const longlong2*>(&R[row * Gm::SR + x])[1];
-    epi.vec4(row0 + (size_t)row * N + x,
+    if constexpr (EpiRaw<Epi>::value)
+      epi.vec4(row0 + (size_t)row * N + x, V4<fx>{{fx{a.x}, fx{a.y}, fx{b.x}, fx{b.y}}}, E, acc);
+    else
+      epi.vec4(row0 + (size_t)row * N + x,
              V4<double>{{value(a.x), value(a.y), value(b.x), value(b.y)}}, acc);
   }
   if constexpr (Epi::NV > 0) block_reduce_finish_acc<Epi::NV, Epi::MAXMASK>(acc, ra, fin);

@@ -109,19 +109,6 @@ __global__ void k_gauss_multiplier(double* __restrict__ M, int nm2, int n, doubl
     M[i] = exp(-0.5 * kf * kf * (double)i * radius * radius) / n3;
 }
 
-// y (FP64) from float-float transforms
-struct EpiStoreFF {
-  static constexpr int NV = 0;
-  static constexpr unsigned MAXMASK = 0;
-  using Acc = AccD;
-  double* out;
-  __device__ void prefetch(size_t, unsigned) const {}
-  __device__ void vec4(size_t i, const V4<ff>& y, Acc*) const {
-    st4(out + i, V4<double>{{to_double(y.v[0]), to_double(y.v[1]), to_double(y.v[2]),
-                            to_double(y.v[3])}});
-  }
-};
-
 }  // namespace
 
 void compare_fields(plc_ctx* c, const double* a, const double* b, double out[4]) {
@@ -182,10 +169,7 @@ void gaussian_smooth(plc_ctx* c, const double* x, double* y, double radius, doub
         table, nm2, c->n, c->box, radius);
     check(cudaGetLastError(), "k_gauss_multiplier");
   }
-  // float-float transforms where the length has a four-step schedule (FP64
-  // accuracy on the FP32 pipes), FP64 Stockham otherwise
-  if (!run_four_step<ff>(c, ProShiftFF{x, ff(0.f, 0.f)}, EpiStoreFF{y}, FinNone{}, 0, nullptr, S_GXFF,
-                         table))
+  if (!run_fixed(c, ProLoad<double>{x}, EpiStore<double>{y}, FinNone{}, 0, nullptr, S_GXFF, table))
     run_pipeline<double>(c, ProLoad<double>{x}, EpiStore<double>{y}, FinNone{}, 0, nullptr, false,
                          table);
   check(cudaStreamSynchronize(c->stream), "stream synchronize");
