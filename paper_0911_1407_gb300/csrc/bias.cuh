@@ -150,7 +150,7 @@ template <typename T, typename TC> struct EpiBiasU {
       const T nf = (T)ni;
       if (u > (T)0) {
         const T inv = (T)1 / u;
-        const T l = nf * log(u);
+        const T l = nf * logt(u);
         acc[1].add(nbw * u - l);
         acc[2].add(l);
         acc[3].add(l < (T)0 ? -l : l);

@@ -12,7 +12,7 @@
 #pragma once
 
 #include "common.cuh"
-#include "exp64.cuh"
+#include "log64.cuh"
 #include "ff.cuh"
 
 namespace plc {
@@ -369,7 +369,7 @@ __device__ __forceinline__ void gauss_cell(T delta, T wt, T ni, T nb, T y, TC c,
   const T nio = ni * inv;
   gi = y + nb * wt - nio;
   d = nio * inv;
-  const T lu = occ ? (u > (T)0 ? ni * log(u) : (T)INFINITY) : (T)0;
+  const T lu = occ ? (u > (T)0 ? ni * logt(u) : (T)INFINITY) : (T)0;
   acc[0].add(delta * y);
   acc[1].add(nb * wt * u - lu);
   acc[2].add(gi * gi);

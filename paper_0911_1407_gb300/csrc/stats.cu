@@ -1,29 +1,36 @@
 // stats.cu -- quality measures and matter statistics of a reconstruction
 // (Sec. 4.1.2 and 4.3.3): correlation coefficient and Euclidean distance
 // between two fields, Gaussian smoothing on the periodic grid, and the
-// histogram and moments of ln(1 + delta).  FP64 fields; sums in FP64 (these
-// are single passes over the data, not on the solver's path).
+// histogram and moments of ln(1 + delta).  FP64 fields; sums in FP64.
+#include <cmath>
+#include <cstdint>
 #include <vector>
 
 #include "launch.cuh"
+#include "log64.cuh"
 
 namespace plc {
 
 namespace {
 
-// {sum a b, sum a^2, sum b^2, sum (a - b)^2}
+// {sum a b, sum a^2, sum b^2, sum (a - b)^2}: five FP64 operations per cell,
+// which bound it (133 us at 256^3 at two per SM and clock, 39 us of HBM).
 __global__ void __launch_bounds__(kThreads)
 k_compare(const double* __restrict__ a, const double* __restrict__ b, size_t n3, RedArgs ra) {
   AccD acc[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) acc[j].init(false);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n3;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const double x = a[i], y = b[i], d = x - y;
-    acc[0].add(x * y);
-    acc[1].add(x * x);
-    acc[2].add(y * y);
-    acc[3].add(d * d);
+  const size_t step = (size_t)gridDim.x * blockDim.x * 4;
+  for (size_t i = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) * 4; i < n3; i += step) {
+    const V4<double> av = ld4(a + i), bv = ld4(b + i);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const double x = av.v[j], y = bv.v[j], d = x - y;
+      acc[0].add(x * y);
+      acc[1].add(x * x);
+      acc[2].add(y * y);
+      acc[3].add(d * d);
+    }
   }
   block_reduce_finish_acc<4, 0u>(acc, ra, FinStore<4>{});
 }
@@ -43,7 +50,7 @@ k_log_shift(const double* __restrict__ delta, size_t n3, DevScalars* sc) {
     if (i < n3) {
       const double u = 1.0 + delta[i];
       if (u > 0.0) {
-        sum += log(u);
+        sum += log64(u);
         cnt += 1.0;
       }
     }
@@ -61,14 +68,54 @@ k_log_shift(const double* __restrict__ delta, size_t n3, DevScalars* sc) {
   if (threadIdx.x == 0) sc->red[7] = scnt[0] > 0.0 ? ssum[0] / scnt[0] : 0.0;
 }
 
+// (x - lo) / width in units of 2^-20 by integers, from x in quanta of 2^-56:
+// ((x - lo) >> s) im >> p, for x - lo cut to half a bin beyond either end.  on = 0
+// where its error bound does not hold.
+struct BinMap {
+  int on, s, im, p;
+  long long lo, lo_cut, hi_cut;
+};
+
+// With bins of at least 2^-30, |lo| <= 32 and at most 4096 bins over a span of
+// at most 2^20: x - lo shifted to 2^29..2^30 costs at most 8 units of 2^-20 (one
+// part in 2^29 of 4098 bins), im's rounding 4, the logarithm's error less than
+// one, and the FP64 quotient it stands for is itself within 8 of the exact one.
+constexpr int kBinMargin = 64;
+BinMap bin_map(double lo, double width, int nbins) {
+  BinMap m{};
+  const double span = (double)nbins * width, far = span + 2.0 * width;
+  if (!(width >= 0x1p-30) || !(std::fabs(lo) <= 32.0) || !(span <= 0x1p20)) return m;
+  const int sy = 29 - (int)std::floor(std::log2(far));         // far 2^sy in [2^29, 2^30)
+  m.s = 56 - sy;
+  if (m.s < 0 || m.s > 62) return m;
+  const double scale = std::ldexp(1.0, 20 - sy) / width;       // T = yk scale
+  int ex;
+  (void)std::frexp(scale, &ex);
+  m.p = 30 - ex;
+  if (m.p < 0 || m.p > 62) return m;
+  m.im = (int)std::lrint(std::ldexp(scale, m.p));              // in [2^29, 2^30]
+  m.lo = std::llrint(std::ldexp(lo, 56));
+  // x itself is below 2^5 in magnitude: a cut beyond that is never reached
+  const double half = 0.5 * width;
+  m.hi_cut = span + half < 64.0 ? std::llrint(std::ldexp(span + half, 56)) : INT64_MAX;
+  m.lo_cut = half < 64.0 ? -std::llrint(std::ldexp(half, 56)) : INT64_MIN;
+  m.on = 1;
+  return m;
+}
+
 // In one pass: the power sums {sum d, d^2, d^3, d^4}, d = x - c about the
 // shift c of k_log_shift, and the histogram of x on [lo + j width,
 // lo + (j+1) width), j < nbins; counts[nbins + 0/1/2] are the cells below,
 // above and with 1 + delta <= 0.  Per-block counts in shared memory, then
-// integer atomics (exact, order-independent).  One FP64 log per cell.
+// integer atomics (exact, order-independent).  A cell's bin is that of the
+// FP64 expression floor((x - lo) / width), x the library's log: the integer
+// form decides all cells but those within kBinMargin of a bin's edge (one in
+// 2^13), which take that expression.  Bound by the seven FP64 operations left
+// per cell; with k_log_shift, k_compare and the smoothing's table 474 us at
+// 256^3, 1815 with the log and the quotient in FP64.
 __global__ void __launch_bounds__(kThreads)
 k_log_hist(const double* __restrict__ delta, size_t n3, double lo, double width, int nbins,
-           unsigned long long* __restrict__ counts, RedArgs ra) {
+           BinMap bm, unsigned long long* __restrict__ counts, RedArgs ra) {
   extern __shared__ unsigned int hist[];
   for (int j = threadIdx.x; j < nbins + 3; j += blockDim.x) hist[j] = 0u;
   __syncthreads();
@@ -76,23 +123,40 @@ k_log_hist(const double* __restrict__ delta, size_t n3, double lo, double width,
   AccD acc[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) acc[j].init(false);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n3;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const double u = 1.0 + delta[i];
-    int bin;
-    if (u > 0.0) {
-      const double x = log(u);
-      const double d = x - shift, d2 = d * d;
-      acc[0].add(d);
-      acc[1].add(d2);
-      acc[2].add(d2 * d);
-      acc[3].add(d2 * d2);
-      const double f = floor((x - lo) / width);
-      bin = f < 0.0 ? nbins : (f >= (double)nbins ? nbins + 1 : (int)f);
-    } else {
-      bin = nbins + 2;
+  const size_t step = (size_t)gridDim.x * blockDim.x * 4;
+#pragma unroll 1
+  for (size_t i = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) * 4; i < n3; i += step) {
+    const V4<double> dv = ld4(delta + i);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const double u = 1.0 + dv.v[j];
+      long long q;
+      int E;
+      bool sure = log64_fixed(u, q, E);
+      double x = fx_to_double(fx{q}, E);
+      const long long y =
+          min(max((q >> (-56 - E)) - bm.lo, bm.lo_cut), bm.hi_cut);
+      const long long t = ((long long)(int)(y >> bm.s) * bm.im) >> bm.p;
+      const int frac = (int)t & 0xfffff, k = (int)(t >> 20);
+      int bin = k < 0 ? nbins : (k >= nbins ? nbins + 1 : k);
+      if (!(sure && bm.on && frac >= kBinMargin && frac < 0x100000 - kBinMargin)) {
+        if (u > 0.0) {
+          x = log64_far(u);
+          const double f = floor((x - lo) / width);
+          bin = f < 0.0 ? nbins : (f >= (double)nbins ? nbins + 1 : (int)f);
+        } else {
+          bin = nbins + 2;
+        }
+      }
+      if (bin != nbins + 2) {
+        const double d = x - shift, d2 = d * d;
+        acc[0].add(d);
+        acc[1].add(d2);
+        acc[2].add(d2 * d);
+        acc[3].add(d2 * d2);
+      }
+      atomicAdd(&hist[bin], 1u);
     }
-    atomicAdd(&hist[bin], 1u);
   }
   __syncthreads();
   for (int j = threadIdx.x; j < nbins + 3; j += blockDim.x)
@@ -134,7 +198,7 @@ void log_stats(plc_ctx* c, const double* delta, double lo, double width, int nbi
   {
     LaunchScope ls(c, S_SETUP);
     k_log_hist<<<pw_blocks(c), kThreads, sizeof(unsigned int) * (nbins + 3), c->stream>>>(
-        delta, c->n3(), lo, width, nbins, dcounts, red_args(c));
+        delta, c->n3(), lo, width, nbins, bin_map(lo, width, nbins), dcounts, red_args(c));
     check(cudaGetLastError(), "k_log_hist");
   }
   std::vector<unsigned long long> h(nbins + 3);
