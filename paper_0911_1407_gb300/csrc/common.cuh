@@ -197,40 +197,37 @@ __device__ __forceinline__ void fft_lines(cpx<T>*& a, cpx<T>*& b, const FftPlan&
 // Register-resident small DFTs (the building blocks of the four-step line
 // transforms in passes4.cuh).
 //
-// exp(2 pi i m / R) for the radices used in registers (R in {2,3,4,6,8,12,16});
+// exp(2 pi i m / R) for the radices used in registers (R in {2,3,4,6,8,12,16,32});
 // after unrolling m and R are constants and the switch folds away.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double unit_cos(int R, int m) {
+__device__ __forceinline__ double cos_12th(int m) {   // cos(2 pi m / 12), 0 <= m < 12
+  const double t = 0.86602540378443864676;
+  switch (m) {
+    case 0: return 1.0; case 1: return t; case 2: return 0.5; case 3: return 0.0;
+    case 4: return -0.5; case 5: return -t; case 6: return -1.0; case 7: return -t;
+    case 8: return -0.5; case 9: return 0.0; case 10: return 0.5; default: return t;
+  }
+}
+__device__ __forceinline__ double cos_32nd(int m) {   // cos(2 pi m / 32), 0 <= m < 32
   const double c1 = 0.92387953251128675613, s1 = 0.38268343236508977173;
-  const double h = 0.70710678118654752440, t = 0.86602540378443864676;
-  if (R == 16) {
-    switch (m & 15) {
-      case 0: return 1.0; case 1: return c1; case 2: return h; case 3: return s1;
-      case 4: return 0.0; case 5: return -s1; case 6: return -h; case 7: return -c1;
-      case 8: return -1.0; case 9: return -c1; case 10: return -h; case 11: return -s1;
-      case 12: return 0.0; case 13: return s1; case 14: return h; default: return c1;
-    }
+  const double h = 0.70710678118654752440;
+  const double o1 = 0.98078528040323044913, o3 = 0.83146961230254523708;   // odd 16ths of pi
+  const double o5 = 0.55557023301960222474, o7 = 0.19509032201612826785;
+  switch (m) {
+    case 0: return 1.0; case 1: case 31: return o1; case 2: case 30: return c1;
+    case 3: case 29: return o3; case 4: case 28: return h; case 5: case 27: return o5;
+    case 6: case 26: return s1; case 7: case 25: return o7; case 8: case 24: return 0.0;
+    case 9: case 23: return -o7; case 10: case 22: return -s1; case 11: case 21: return -o5;
+    case 12: case 20: return -h; case 13: case 19: return -o3; case 14: case 18: return -c1;
+    case 15: case 17: return -o1; default: return -1.0;
   }
-  if (R == 12) {
-    switch (m % 12) {
-      case 0: return 1.0; case 1: return t; case 2: return 0.5; case 3: return 0.0;
-      case 4: return -0.5; case 5: return -t; case 6: return -1.0; case 7: return -t;
-      case 8: return -0.5; case 9: return 0.0; case 10: return 0.5; default: return t;
-    }
-  }
-  if (R == 8) return unit_cos(16, 2 * m);
-  if (R == 6) return unit_cos(12, 2 * m);
-  if (R == 4) return unit_cos(16, 4 * m);
-  if (R == 3) return unit_cos(12, 4 * m);
-  return (m & 1) ? -1.0 : 1.0;   // R == 2
+}
+// m non-negative; sin(x) = cos(x - pi/2)
+__device__ __forceinline__ double unit_cos(int R, int m) {
+  return R % 3 == 0 ? cos_12th(m * (12 / R) % 12) : cos_32nd(m * (32 / R) & 31);
 }
 __device__ __forceinline__ double unit_sin(int R, int m) {
-  // sin(2 pi m / R) = cos(2 pi (m - R/4) / R) for R divisible by 4; the
-  // radices 6 and 3 go through 12
-  if (R == 6) return unit_sin(12, 2 * m);
-  if (R == 3) return unit_sin(12, 4 * m);
-  if (R == 2) return 0.0;
-  return unit_cos(R, ((m - R / 4) % R + R) % R);
+  return R % 3 == 0 ? cos_12th((m * (12 / R) + 9) % 12) : cos_32nd((m * (32 / R) + 24) & 31);
 }
 
 // a * exp(SIGN 2 pi i m / R)
@@ -247,8 +244,8 @@ template <typename T, int SIGN> struct Rot {
   }
 };
 
-// In-register DFT of length R (natural order in and out).  R = 6, 12, 16 are
-// done four-step as R1 x R2 (2x3, 3x4, 4x4).
+// In-register DFT of length R (natural order in and out).  R = 6, 12, 16, 32
+// are done four-step as R1 x R2 (2x3, 3x4, 4x4, 4x8).
 template <typename T, int SIGN, int R>
 __device__ __forceinline__ void dft_small(cpx<T>* v) {
   using C = cpx<T>;

@@ -35,15 +35,19 @@ enum Site {
 extern const char* const kSiteNames[S_NSITES];
 
 // Line-transform schedules with a register four-step form: n = f1 f2
-// (passes4.cuh in FP32, passesx.cuh for FP64 fields, which takes the first
-// entry of its n whichever is set).  The first entry for an n is the default;
+// (passes4.cuh in FP32; passesx.cuh for FP64 fields of a fixed_length, which
+// takes the first entry of its n whichever is set).  The first entry for an n is the default;
 // plc_autotune times every FP32 entry for n and the Stockham form
 // (f1 = f2 = 0).
 struct FourStepShape {
   int n, f1, f2;
 };
+// Lengths with fixed-point FP64 passes.
+constexpr bool fixed_length(int n) {
+  return n == 256 || n == 192 || n == 128 || n == 96 || n == 64 || n == 32;
+}
 constexpr FourStepShape kFourStep[] = {
-    {256, 16, 16}, {192, 16, 12}, {192, 12, 16}, {128, 16, 8}, {128, 8, 16},
+    {512, 32, 16}, {256, 16, 16}, {192, 16, 12}, {192, 12, 16}, {128, 16, 8}, {128, 8, 16},
     {96, 12, 8},   {96, 8, 12},   {64, 8, 8},    {32, 8, 4}};
 
 struct Profiler {

@@ -452,10 +452,7 @@ void capture_solve(plc_ctx* c, cudaGraph_t top, const std::vector<cudaStream_t>&
   // the switch's sums-only check: mixed solves of lengths with fixed-point
   // transforms (a four-step schedule)
   bool has_check = false;
-  if constexpr (kMixed) {
-    for (const FourStepShape& q : kFourStep)
-      if (q.n == c->n && q.f1 == c->plan.f1 && q.f2 == c->plan.f2) has_check = true;
-  }
+  if constexpr (kMixed) has_check = c->plan.f1 != 0 && fixed_length(c->n);
   if (has_check) {
     mk(&h_full);
     mk(&h_chk);

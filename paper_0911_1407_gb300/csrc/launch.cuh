@@ -85,6 +85,7 @@ template <typename T, typename Pro, typename Epi, typename Fin>
 bool run_four_step(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* done, int s0,
                    const T* m_override = nullptr) {
   switch (c->plan.f1 * 64 + c->plan.f2) {
+    case 32 * 64 + 16: run_pipeline4<T, 32, 16>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
     case 16 * 64 + 16: run_pipeline4<T, 16, 16>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
     case 16 * 64 + 12: run_pipeline4<T, 16, 12>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
     case 12 * 64 + 16: run_pipeline4<T, 12, 16>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
@@ -145,7 +146,7 @@ void run_pipelinex(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int
 template <typename Pro, typename Epi, typename Fin>
 bool run_fixed(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* done, int s0,
                const double* m_override) {
-  if (!c->plan.f1) return false;
+  if (!c->plan.f1 || !fixed_length(c->n)) return false;
   switch (c->n) {
     case 256: run_pipelinex<16, 16>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;
     case 192: run_pipelinex<16, 12>(c, pro, epi, fin, zero_dc, done, s0, m_override); return true;

@@ -3,7 +3,7 @@
 //
 // Same pipeline and global layouts as passes.cuh (XF -> A[z][kx][y] -> YF ->
 // B[kx][ky][z] -> Z -> YI -> A -> XI), for n = N1 N2 with (N1, N2) in
-// {(16,16), (16,12), (16,8), (12,8), (8,8), (8,4)}.  A line of length N is
+// {(32,16), (16,16), (16,12), (16,8), (12,8), (8,8), (8,4)}.  A line of length N is
 // transformed in two register phases joined by one shared-memory exchange:
 //
 //   forward  Z[k1 + N1 k2] = sum_n2 W_N2^{n2 k2} W_N^{n2 k1}
@@ -62,7 +62,14 @@ template <typename T, int N1_, int N2_> struct Geo4 {
   static constexpr size_t smem_z = tw_bytes + x_bytes + m_bytes;
   static constexpr size_t smem_x = tw_bytes + (x_bytes > r_bytes ? x_bytes : r_bytes);
   static_assert(L * N2 <= kThreads, "one phase-A task per thread at most");
-  static_assert(N1 / 2 <= kThreads / 32, "one warp per pair of x-pass tasks");
+};
+
+// Resident blocks per SM asked of the compiler by a pass with a register DFT
+// of length 32 (it takes more than 128 registers unbounded, one block per
+// SM).  Shorter ones are left to the compiler, the y passes without a block
+// count (0; a count of 1 takes the y-inverse from 48 to 66 registers).
+template <int N1, int SHORT> struct MinBlocks4 {
+  static constexpr int value = N1 > 16 ? 2 : SHORT;
 };
 
 // tw2[k1 N2 + n2] = W_N^{k1 n2} from the natural table tw[m] = W_N^m.
@@ -116,7 +123,7 @@ __device__ __forceinline__ void phase_b_inv(cpx<T>* v, const cpx<T>* tw2, int k1
 // without its guard or task loop.
 // ---------------------------------------------------------------------------
 template <typename T, int N1, int N2>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, MinBlocks4<N1, 0>::value)
 k4_yf(const cpx<T>* __restrict__ A, cpx<T>* __restrict__ B, const cpx<T>* __restrict__ twg,
       const int* __restrict__ done) {
   PLC_PASS4_SETUP(C* X = tw2 + N);
@@ -165,6 +172,7 @@ k4_yf(const cpx<T>* __restrict__ A, cpx<T>* __restrict__ B, const cpx<T>* __rest
 // without a block count does (a count of 1 changes it).
 template <typename T, int N1, int N2> struct ZMinBlocks { static constexpr int value = 0; };
 template <> struct ZMinBlocks<float, 16, 16> { static constexpr int value = 3; };
+template <> struct ZMinBlocks<float, 32, 16> { static constexpr int value = 2; };
 
 // ---------------------------------------------------------------------------
 // Z: forward c2c along z, times M[|m|^2] = 1/(lambda_k n^3), inverse c2c,
@@ -252,7 +260,7 @@ k4_z(cpx<T>* __restrict__ B, const T* __restrict__ M, int zero_dc,
 // B[kx][:][z0 + c] and writes A[z0 + c][kx][:].
 // ---------------------------------------------------------------------------
 template <typename T, int N1, int N2>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, MinBlocks4<N1, 0>::value)
 k4_yi(const cpx<T>* __restrict__ B, cpx<T>* __restrict__ A, const cpx<T>* __restrict__ twg,
       const int* __restrict__ done) {
   PLC_PASS4_PROLOGUE(C* X = tw2 + N);
@@ -321,7 +329,7 @@ template <typename Pro> struct XfBatch<Pro, decltype((void)Pro::kBatch)> {
 };
 
 template <typename T, int N1, int N2, typename Pro>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, MinBlocks4<N1, 1>::value)
 k4_xf(Pro pro, cpx<T>* __restrict__ A, const cpx<T>* __restrict__ twg,
       const int* __restrict__ done) {
   PLC_PASS4_SETUP(T* R = reinterpret_cast<T*>(tw2 + N); C* X = tw2 + N);
@@ -369,8 +377,8 @@ k4_xf(Pro pro, cpx<T>* __restrict__ A, const cpx<T>* __restrict__ twg,
   }
   __syncthreads();
   // phase B in pairs k1, N1 - k1 (one warp per pair), split into X_a, X_b
-  const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (g < N1 / 2) {
+  const int lane = threadIdx.x & 31;
+  auto pair_b = [&](int g) {
     const int c = lane & 15, member = lane >> 4;
     const int k1 = pair_k1<N1>(g, member);
 #pragma unroll
@@ -399,6 +407,11 @@ k4_xf(Pro pro, cpx<T>* __restrict__ A, const cpx<T>* __restrict__ twg,
 #pragma unroll
       for (int k2 = 0; k2 < N2 / 2; ++k2) put(k2, v[k2], v[N2 - 1 - k2]);
     }
+  };
+  if constexpr (N1 / 2 <= kThreads / 32) {
+    if (threadIdx.x >> 5 < N1 / 2) pair_b(threadIdx.x >> 5);
+  } else {
+    for (int g = threadIdx.x >> 5; g < N1 / 2; g += kThreads / 32) pair_b(g);
   }
 }
 
@@ -420,7 +433,7 @@ template <typename Epi> struct EpiUnroll<Epi, decltype((void)Epi::kUnroll)> {
 // and accumulates Epi::NV sums; Fin runs once on the grid totals.
 // ---------------------------------------------------------------------------
 template <typename T, int N1, int N2, typename Epi, typename Fin>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, MinBlocks4<N1, 1>::value)
 k4_xi(const cpx<T>* __restrict__ A, Epi epi, Fin fin, RedArgs ra,
       const cpx<T>* __restrict__ twg, const int* __restrict__ done) {
   PLC_PASS4_PROLOGUE(T* R = reinterpret_cast<T*>(tw2 + N); C* X = tw2 + N);
@@ -429,9 +442,9 @@ k4_xi(const cpx<T>* __restrict__ A, Epi epi, Fin fin, RedArgs ra,
   // the epilogue's operands do not depend on the transform: request them
   // into L2 now, so that their latency hides behind the transform
   if (threadIdx.x == 0) epi.prefetch(row0, Gm::RY * N);
-  const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
   C v[N1 > N2 ? N1 : N2];
-  if (g < N1 / 2) {
+  auto pair_b = [&](int g) {
     const int c = lane & 15, member = lane >> 4;
     const int k1 = pair_k1<N1>(g, member);
     const C* src = A + ((size_t)z * h + k1) * N + y0 + 2 * c;
@@ -466,6 +479,11 @@ k4_xi(const cpx<T>* __restrict__ A, Epi epi, Fin fin, RedArgs ra,
     phase_b_inv<T, N1, N2>(v, tw2, k1);
 #pragma unroll
     for (int n2 = 0; n2 < N2; ++n2) X[c * Gm::S + k1 * N2 + n2] = v[n2];
+  };
+  if constexpr (N1 / 2 <= kThreads / 32) {
+    if (threadIdx.x >> 5 < N1 / 2) pair_b(threadIdx.x >> 5);
+  } else {
+    for (int g = threadIdx.x >> 5; g < N1 / 2; g += kThreads / 32) pair_b(g);
   }
   __syncthreads();
   const bool task_a = threadIdx.x < Gm::L * N2;

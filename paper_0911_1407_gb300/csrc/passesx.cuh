@@ -25,6 +25,7 @@
 // 128^3 / 192^3 / 256^3 went from 327 / 1170 / 3450 us to 88 / 263 / 480.
 #pragma once
 
+#include "ctx.h"
 #include "fx.cuh"
 #include "passes4.cuh"
 
@@ -52,6 +53,8 @@ inline FxExps fx_exps(int* p, int n) {
 constexpr int kFxBlocks = 2;
 
 template <int N1_, int N2_> struct GeoX : Geo4<fx, N1_, N2_> {
+  static_assert(N1_ / 2 <= kThreads / 32, "one warp per pair of x-pass tasks");
+  static_assert(fixed_length(N1_ * N2_), "listed as a fixed-point length");
   using G = Geo4<fx, N1_, N2_>;
   static constexpr int NM = N1_ > N2_ ? N1_ : N2_;
   // per-thread L1 parts: line c at [c * (NM + 1)]
