@@ -385,38 +385,65 @@ __device__ __forceinline__ double red_identity(int j) {
   return ((MAXMASK >> j) & 1u) ? -INFINITY : 0.0;
 }
 
+// Reduce the 256 threads' v[NV] in a fixed order; thread 0 gets the results
+// (in v, after the barrier that ends this).  The order is that of shuffles by
+// 16, 8, 4, 2, 1 within each warp and 4, 2, 1 across the eight warps, but one
+// warp does each value's whole tree with its lanes full: 12 additions in place
+// of 40 to 45 half-empty ones.  A warp's FP64 instruction takes 16 clocks of the SM's
+// FP64 pipe however many of its lanes are active, and the plain shuffles of
+// three values took 2 us of pipe time in the last block of every reduction,
+// while the GPU waited.  live: warps beyond it hold only identities.
 template <int NV, unsigned MAXMASK>
-__device__ __forceinline__ void warp_reduce(double* v) {
+__device__ __forceinline__ void block_tree(double* v, double (*sh)[kThreads], int live) {
+  static_assert(NV <= kThreads / 32, "one warp per value");
+  __shared__ double res[NV];
+  const int t = threadIdx.x, l = t & 31, j = t >> 5;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int q = 0; q < NV; ++q) sh[q][t] = v[q];
+  __syncthreads();
+  if (j < NV) {
+    const bool mx = (MAXMASK >> j) & 1u;
+    auto op = [&](double a, double b) { return mx ? fmax(a, b) : a + b; };
+    const double id = mx ? -INFINITY : 0.0;
+    // by 16: lane (bit 4, i) holds the pairs i, i + 16 of warps 2k + bit 4
+    double a[4];
 #pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] = red_op<MAXMASK>(j, v[j], __shfl_down_sync(0xffffffffu, v[j], o));
+    for (int k = 0; k < 4; ++k) {
+      a[k] = id;
+      if (2 * k < live) {
+        const double* w = &sh[j][32 * (2 * k + (l >> 4)) + (l & 15)];
+        a[k] = op(w[0], w[16]);
+      }
+    }
+    // by 8: lanes with bit 3 clear go on with k = 0, 1, the others with 2, 3
+    const bool b3 = l & 8, b2 = l & 4;
+    const double s0 = __shfl_xor_sync(0xffffffffu, b3 ? a[0] : a[2], 8);
+    const double s1 = __shfl_xor_sync(0xffffffffu, b3 ? a[1] : a[3], 8);
+    const double c0 = op(b3 ? a[2] : a[0], s0);
+    double c1 = b3 ? a[3] : a[1];
+    if (live > 2) c1 = op(c1, s1);
+    // by 4: bit 2 takes the other k of its pair
+    const double s2 = __shfl_xor_sync(0xffffffffu, b2 ? c0 : c1, 4);
+    double d = op(b2 ? c1 : c0, s2);
+    d = op(d, __shfl_xor_sync(0xffffffffu, d, 2));
+    d = op(d, __shfl_xor_sync(0xffffffffu, d, 1));
+    // warp of this lane's sum: 4 bit 3 + 2 bit 2 + bit 4
+    if (live > 4) d = op(d, __shfl_xor_sync(0xffffffffu, d, 8));
+    if (live > 2) d = op(d, __shfl_xor_sync(0xffffffffu, d, 4));
+    d = op(d, __shfl_xor_sync(0xffffffffu, d, 16));
+    if (l == 0) res[j] = d;
   }
-}
-
-// Reduce v[NV] over the block in a fixed order; thread 0 gets the result.
-template <int NV, unsigned MAXMASK>
-__device__ __forceinline__ void block_reduce(double* v, double* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nw = blockDim.x >> 5;
-  warp_reduce<NV, MAXMASK>(v);
   __syncthreads();
-  if (lane == 0)
+  if (t == 0)
 #pragma unroll
-    for (int j = 0; j < NV; ++j) sh[warp * NV + j] = v[j];
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] = lane < nw ? sh[lane * NV + j] : red_identity<MAXMASK>(j);
-    warp_reduce<NV, MAXMASK>(v);
-  }
-  __syncthreads();
+    for (int q = 0; q < NV; ++q) v[q] = res[q];
 }
 
 // The grid reduction behind block_reduce_finish: v (thread 0's block
 // totals) to the partials; the last block sums them in block order.
 template <int NV, unsigned MAXMASK, typename Fin>
-__device__ __forceinline__ void grid_finish(double* v, const RedArgs& ra, Fin fin, double* sh) {
+__device__ __forceinline__ void grid_finish(double* v, const RedArgs& ra, Fin fin,
+                                            double (*sh)[kThreads]) {
   __shared__ int is_last;
   const unsigned nblocks = gridDim.x * gridDim.y * gridDim.z;
   const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
@@ -430,41 +457,47 @@ __device__ __forceinline__ void grid_finish(double* v, const RedArgs& ra, Fin fi
   __syncthreads();
   if (!is_last) return;
   __threadfence();
+  // the scalars fin reads, on their way while the partials are summed
+  if (threadIdx.x < sizeof(DevScalars) / 32)
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(reinterpret_cast<const char*>(ra.sc) + 32 * threadIdx.x));
   double acc[NV];
 #pragma unroll
   for (int j = 0; j < NV; ++j) acc[j] = red_identity<MAXMASK>(j);
   // U partials per thread loaded before they are summed (in the same
   // order, b = tid, tid + blockDim, ...), so that the last block waits for
   // about one L2 round trip per U instead of one per partial: this runs
-  // while the rest of the GPU waits for the kernel to end
+  // while the rest of the GPU waits for the kernel to end.  A warp beyond the
+  // partials adds nothing (the additions cost FP64 pipe time).
   constexpr int U = NV <= 1 ? 8 : (NV <= 3 ? 4 : 2);
-  for (unsigned b0 = threadIdx.x; b0 < nblocks; b0 += U * blockDim.x) {
+  const unsigned wbase = threadIdx.x & ~31u;
+  for (unsigned b0 = 0; b0 < nblocks; b0 += U * kThreads) {
     double t[U][NV];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const unsigned b = b0 + u * blockDim.x;
+      const unsigned b = b0 + u * kThreads + threadIdx.x;
 #pragma unroll
       for (int j = 0; j < NV; ++j)
         t[u][j] = b < nblocks ? __ldcg(ra.partials + (size_t)b * kMaxRed + j) : red_identity<MAXMASK>(j);
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+    for (int u = 0; u < U; ++u) {
+      if (b0 + u * kThreads + wbase >= nblocks) break;
 #pragma unroll
       for (int j = 0; j < NV; ++j) acc[j] = red_op<MAXMASK>(j, acc[j], t[u][j]);
+    }
   }
-  block_reduce<NV, MAXMASK>(acc, sh);
+  block_tree<NV, MAXMASK>(acc, sh, (int)min((nblocks + 31u) / 32u, 8u));
   if (threadIdx.x == 0) {
     fin(acc, ra.sc);
     ra.sc->ticket = 0u;
-    __threadfence();
   }
 }
 
 // Deterministic grid reduction of per-thread FP64 values v[NV].
 template <int NV, unsigned MAXMASK, typename Fin>
 __device__ __forceinline__ void block_reduce_finish(double* v, const RedArgs& ra, Fin fin) {
-  __shared__ double sh[32 * kMaxRed];
-  block_reduce<NV, MAXMASK>(v, sh);
+  __shared__ double sh[NV][kThreads];
+  block_tree<NV, MAXMASK>(v, sh, kThreads / 32);
   grid_finish<NV, MAXMASK>(v, ra, fin, sh);
 }
 
@@ -473,33 +506,38 @@ __device__ __forceinline__ void block_reduce_finish(double* v, const RedArgs& ra
 // go to FP64 once.
 template <int NV, unsigned MAXMASK, typename Acc, typename Fin>
 __device__ __forceinline__ void block_reduce_finish_acc(Acc* a, const RedArgs& ra, Fin fin) {
-  __shared__ Acc sa[32 * kMaxRed];
-  __shared__ double sh[32 * kMaxRed];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int j = 0; j < NV; ++j) a[j].merge(a[j].shfl_down(o), (MAXMASK >> j) & 1u);
-  if (lane == 0)
-#pragma unroll
-    for (int j = 0; j < NV; ++j) sa[warp * NV + j] = a[j];
-  __syncthreads();
+  __shared__ double sh[NV][kThreads];
   double v[NV];
-  if (warp == 0) {
+  if constexpr (std::is_same<Acc, AccD>::value) {
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      if (lane < nw) a[j] = sa[lane * NV + j];
-      else a[j].init((MAXMASK >> j) & 1u);
-    }
+    for (int j = 0; j < NV; ++j) v[j] = a[j].get();
+    block_tree<NV, MAXMASK>(v, sh, kThreads / 32);
+  } else {
+    __shared__ Acc sa[kThreads / 32 * NV];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kThreads / 32;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
       for (int j = 0; j < NV; ++j) a[j].merge(a[j].shfl_down(o), (MAXMASK >> j) & 1u);
-  }
-  if (threadIdx.x == 0)
+    if (lane == 0)
 #pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] = a[j].get();
-  __syncthreads();
+      for (int j = 0; j < NV; ++j) sa[warp * NV + j] = a[j];
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+      for (int j = 0; j < NV; ++j) {
+        if (lane < nw) a[j] = sa[lane * NV + j];
+        else a[j].init((MAXMASK >> j) & 1u);
+      }
+#pragma unroll
+      for (int o = nw / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int j = 0; j < NV; ++j) a[j].merge(a[j].shfl_down(o), (MAXMASK >> j) & 1u);
+    }
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int j = 0; j < NV; ++j) v[j] = a[j].get();
+  }
   grid_finish<NV, MAXMASK>(v, ra, fin, sh);
 }
 

@@ -30,9 +30,9 @@ template <typename T, auto Kernel> inline void set_smem() {
 
 inline RedArgs red_args(plc_ctx* c) { return RedArgs{c->partials, c->sc}; }
 
-// Raise a kernel's dynamic shared-memory limit once (when above 48 KB).
+// Raise a kernel's dynamic shared-memory limit once (also below 48 KB, which
+// is the limit for its static and dynamic shared memory together).
 template <auto Kernel> inline void set_smem4(size_t bytes) {
-  if (bytes <= 48 * 1024) return;
   static const cudaError_t once =
       cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   check(once, "cudaFuncSetAttribute");
