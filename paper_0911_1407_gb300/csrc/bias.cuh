@@ -34,7 +34,6 @@ template <typename T> struct ProExpm1 {
   const T* s;
   __device__ void prepare() {}
   __device__ void prefetch(size_t i, unsigned cnt) const { prefetch_l2(s + i, cnt * sizeof(T)); }
-  __device__ T operator()(size_t i) const { return expm1(__ldg(s + i)); }
   __device__ V4<T> vec4(size_t i) const {
     V4<T> a = ld4(s + i);
 #pragma unroll
@@ -53,11 +52,6 @@ template <typename T, typename TC> struct ProTrial {
   __device__ void prefetch(size_t i, unsigned cnt) const {
     prefetch_l2(s + i, cnt * sizeof(T));
     prefetch_l2(xi + i, cnt * sizeof(TC));
-  }
-  __device__ T operator()(size_t i) const {
-    const T sn = __ldg(s + i) + tau * (T)__ldg(xi + i);
-    s2[i] = sn;
-    return expm1(sn);
   }
   __device__ V4<T> vec4(size_t i) const {
     const V4<T> sv = ld4(s + i);
@@ -82,7 +76,6 @@ template <typename T> struct ProMul {
     prefetch_l2(f + i, cnt * sizeof(T));
     prefetch_l2(v + i, cnt * sizeof(T));
   }
-  __device__ T operator()(size_t i) const { return __ldg(f + i) * __ldg(v + i); }
   __device__ V4<T> vec4(size_t i) const {
     const V4<T> a = ld4(f + i), b = ld4(v + i);
     V4<T> o;
@@ -102,7 +95,6 @@ template <typename T, bool JAC> struct ProCgDirE {
     dir.prefetch(i, cnt);
     prefetch_l2(E + i, cnt * sizeof(T));
   }
-  __device__ T operator()(size_t i) const { return dir(i) * __ldg(E + i); }
   __device__ V4<T> vec4(size_t i) const {
     V4<T> o = dir.vec4(i);
     const V4<T> e = ld4(E + i);

@@ -173,6 +173,55 @@ __device__ __forceinline__ void stockham_stage(const cpx<T>* __restrict__ in,
   }
 }
 
+// The same stage on `nl` lines of any number at line stride sl and element
+// stride se (lines on consecutive threads); nld divides by nl.
+template <typename T, int R, int SIGN>
+__device__ __forceinline__ void stockham_stage_n(const cpx<T>* __restrict__ in,
+                                                 cpx<T>* __restrict__ out, int N, int Ns,
+                                                 unsigned ns_m, int tstep, int nl, FastDiv nld,
+                                                 int sl, int se, const cpx<T>* __restrict__ tw) {
+  using C = cpx<T>;
+  const int NR = N / R;
+  for (int b = threadIdx.x; b < nl * NR; b += blockDim.x) {
+    const int j = fdiv(b, nld), c = b - j * nl;
+    const int k = ns_m ? j - (int)__umulhi((unsigned)j, ns_m) * Ns : 0;
+    C v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = in[(j + r * NR) * se + c * sl];
+    if (k != 0) {
+#pragma unroll
+      for (int r = 1; r < R; ++r) {
+        C w = tw[r * k * tstep];
+        if (SIGN > 0) w.y = -w.y;
+        v[r] = cmul(v[r], w);
+      }
+    }
+    if (R == 2) Dft<T, SIGN>::r2(v);
+    if (R == 3) Dft<T, SIGN>::r3(v);
+    if (R == 4) Dft<T, SIGN>::r4(v);
+    if (R == 8) Dft<T, SIGN>::r8(v);
+    const int d = (j - k) * R + k;
+#pragma unroll
+    for (int r = 0; r < R; ++r) out[(d + r * Ns) * se + c * sl] = v[r];
+  }
+}
+template <typename T, int SIGN>
+__device__ __forceinline__ void fft_lines_n(cpx<T>*& a, cpx<T>*& b, const FftPlan& plan, int nl,
+                                            int sl, int se, const cpx<T>* tw) {
+  const int N = plan.n;
+  const FastDiv nld = nl == N ? plan.nd : make_fastdiv(nl);
+  for (int s = 0; s < plan.nst; ++s) {
+    const int R = plan.rad[s], Ns = plan.ns[s], ts = plan.tstep[s];
+    const unsigned m = plan.ns_m[s];
+    if (R == 8) stockham_stage_n<T, 8, SIGN>(a, b, N, Ns, m, ts, nl, nld, sl, se, tw);
+    else if (R == 4) stockham_stage_n<T, 4, SIGN>(a, b, N, Ns, m, ts, nl, nld, sl, se, tw);
+    else if (R == 2) stockham_stage_n<T, 2, SIGN>(a, b, N, Ns, m, ts, nl, nld, sl, se, tw);
+    else stockham_stage_n<T, 3, SIGN>(a, b, N, Ns, m, ts, nl, nld, sl, se, tw);
+    __syncthreads();
+    cpx<T>* t = a; a = b; b = t;
+  }
+}
+
 // Full length-N transform of `nl` (<= L) lines, ping-ponging between two
 // buffers.  On return `a` points at the result and `b` at the free buffer.
 // Must be entered after a __syncthreads() that publishes the data; ends with

@@ -121,6 +121,10 @@ struct plc_ctx {
   static constexpr int kNumBiasWork = 12;
   void* bwf[kNumBiasWork] = {};
 
+  // set while a batch captures this context's solve: other solves will run
+  // beside it
+  bool shared_chip = false;
+
   plc::Profiler prof;
   std::string err;
 

@@ -618,6 +618,13 @@ struct Streams {
   }
 };
 
+// Marks a context as sharing the chip for the life of this object.
+struct SharedChip {
+  plc_ctx* c;
+  SharedChip(plc_ctx* ctx, bool on) : c(ctx) { c->shared_chip = on; }
+  ~SharedChip() { c->shared_chip = false; }
+};
+
 void fill_stats(const DevCtl& h, plc_stats* st, double ms) {
   if (!st) return;
   std::memset(st, 0, sizeof(*st));
@@ -730,6 +737,7 @@ plc_status batch_map(BatchGraph* b, const std::vector<plc_ctx*>& cs, const int32
     try {
       for (size_t i = 0; i < m; ++i) {
         const double* wi = w ? w[i] : nullptr;
+        const SharedChip sc(cs[i], m > 1);
         if (cs[i]->precision == PLC_FP64)
           capture_solve<double>(cs[i], top, ss.s, N[i], wi, nbar[i], s[i], o);
         else

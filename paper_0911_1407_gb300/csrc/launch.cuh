@@ -51,26 +51,46 @@ void run_pipeline4(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int
   const T* M = m_override ? m_override : multiplier<T>(c);
   const dim3 gx(n / Gm::RY, n), gy(n / Gm::L, h);
   set_smem4<k4_xf<T, N1, N2, Pro>>(Gm::smem_x);
-  set_smem4<k4_yf<T, N1, N2>>(Gm::smem_y);
-  set_smem4<k4_z<T, N1, N2>>(Gm::smem_z);
-  set_smem4<k4_yi<T, N1, N2>>(Gm::smem_y);
   set_smem4<k4_xi<T, N1, N2, Epi, Fin>>(Gm::smem_x);
   {
     LaunchScope ls(c, Site(s0 + 0));
     k4_xf<T, N1, N2, Pro><<<gx, kThreads, Gm::smem_x, c->stream>>>(pro, A, tw, done);
   }
-  {
-    LaunchScope ls(c, Site(s0 + 1));
-    k4_yf<T, N1, N2><<<gy, kThreads, Gm::smem_y, c->stream>>>(A, B, tw, done);
-  }
-  {
-    LaunchScope ls(c, Site(s0 + 2));
-    k4_z<T, N1, N2><<<gy, kThreads, Gm::smem_z, c->stream>>>(B, M, zero_dc, tw, done);
-  }
-  {
-    LaunchScope ls(c, Site(s0 + 3));
-    k4_yi<T, N1, N2><<<gy, kThreads, Gm::smem_y, c->stream>>>(B, A, tw, done);
-  }
+  // The y and z passes of a plane in one block (k4_yzy) up to 96^3: mixed MAP
+  // at 32^3 904 -> 835 us, 64^3 867 -> 832, 96^3 1240 -> 1237.  At 128^3 its 65
+  // planes leave half the chip idle, and a solve by itself is slower (1601 ->
+  // 1645 us), but solves that share the chip gain from the traffic saved
+  // (64 mocks up to 128^3: 37.8 -> 36.2 ms).
+  auto fused = [&]() {
+    if constexpr (n <= 128) {
+      using Gp = GeoP<N1, N2>;
+      constexpr size_t bytes = Gp::template smem<C>();
+      set_smem4<k4_yzy<T, N1, N2>>(bytes);
+      LaunchScope ls(c, Site(s0 + 2));
+      k4_yzy<T, N1, N2><<<h, Gp::kT, bytes, c->stream>>>(A, M, zero_dc, tw, done);
+    }
+  };
+  auto three_passes = [&]() {
+    if constexpr (n > 96) {
+      set_smem4<k4_yf<T, N1, N2>>(Gm::smem_y);
+      set_smem4<k4_z<T, N1, N2>>(Gm::smem_z);
+      set_smem4<k4_yi<T, N1, N2>>(Gm::smem_y);
+      {
+        LaunchScope ls(c, Site(s0 + 1));
+        k4_yf<T, N1, N2><<<gy, kThreads, Gm::smem_y, c->stream>>>(A, B, tw, done);
+      }
+      {
+        LaunchScope ls(c, Site(s0 + 2));
+        k4_z<T, N1, N2><<<gy, kThreads, Gm::smem_z, c->stream>>>(B, M, zero_dc, tw, done);
+      }
+      {
+        LaunchScope ls(c, Site(s0 + 3));
+        k4_yi<T, N1, N2><<<gy, kThreads, Gm::smem_y, c->stream>>>(B, A, tw, done);
+      }
+    }
+  };
+  if (n <= 96 || (n <= 128 && c->shared_chip)) fused();
+  else three_passes();
   {
     LaunchScope ls(c, Site(s0 + 4));
     k4_xi<T, N1, N2, Epi, Fin><<<gx, kThreads, Gm::smem_x, c->stream>>>(A, epi, fin, red_args(c),
@@ -158,6 +178,10 @@ bool run_fixed(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* do
   }
 }
 
+// Shared memory of the Stockham plane kernel: two planes of up to 108^2 FP32
+// modes.  FP64 planes stay apart: n/2+1 blocks would leave most FP64 pipes idle.
+constexpr size_t kPlaneSmem = 200 * 1024;
+
 // The five passes XF -> YF -> Z -> YI -> XI on the context's stream.
 template <typename T, typename Pro, typename Epi, typename Fin>
 void run_pipeline(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* done,
@@ -189,18 +213,25 @@ void run_pipeline(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int*
     LaunchScope ls(c, Site(s0 + 0));
     k_xf<T, Pro><<<gx, kThreads, sm, c->stream>>>(pro, A, c->plan, tw, done);
   }
-  {
-    LaunchScope ls(c, Site(s0 + 1));
-    k_yf<T><<<gy, kThreads, sm, c->stream>>>(A, B, c->plan, tw, done);
-  }
-  {
+  if (sizeof(T) == 4 && plane_smem<T>(n) <= kPlaneSmem) {
+    set_smem4<k_yzy<T>>(kPlaneSmem);
     LaunchScope ls(c, Site(s0 + 2));
-    k_z<T><<<gy, kThreads, sm, c->stream>>>(B, m_override ? m_override : multiplier<T>(c), zero_dc,
-                                            c->plan, tw, done);
-  }
-  {
-    LaunchScope ls(c, Site(s0 + 3));
-    k_yi<T><<<gy, kThreads, sm, c->stream>>>(B, A, c->plan, tw, done);
+    k_yzy<T><<<h, kPlaneThreads, plane_smem<T>(n), c->stream>>>(
+        A, m_override ? m_override : multiplier<T>(c), zero_dc, c->plan, tw, done);
+  } else {
+    {
+      LaunchScope ls(c, Site(s0 + 1));
+      k_yf<T><<<gy, kThreads, sm, c->stream>>>(A, B, c->plan, tw, done);
+    }
+    {
+      LaunchScope ls(c, Site(s0 + 2));
+      k_z<T><<<gy, kThreads, sm, c->stream>>>(B, m_override ? m_override : multiplier<T>(c), zero_dc,
+                                              c->plan, tw, done);
+    }
+    {
+      LaunchScope ls(c, Site(s0 + 3));
+      k_yi<T><<<gy, kThreads, sm, c->stream>>>(B, A, c->plan, tw, done);
+    }
   }
   {
     LaunchScope ls(c, Site(s0 + 4));

@@ -59,7 +59,6 @@ template <typename T> struct ProLoad {
   const T* x;
   __device__ void prepare() {}
   __device__ void prefetch(size_t i, unsigned cnt) const { prefetch_l2(x + i, cnt * sizeof(T)); }
-  __device__ T operator()(size_t i) const { return __ldg(x + i); }
   __device__ V4<T> vec4(size_t i) const { return ld4(x + i); }
 };
 
@@ -71,7 +70,6 @@ template <typename T, typename TS> struct ProShift {
   __device__ void prepare() {}
   __device__ void prefetch(size_t i, unsigned cnt) const { prefetch_l2(s + i, cnt * sizeof(TS)); }
   // difference taken in the transform precision (no FP64 work for float)
-  __device__ T operator()(size_t i) const { return (T)__ldg(s + i) - (T)mu; }
   __device__ V4<T> vec4(size_t i) const {
     const V4<TS> a = ld4(s + i);
     V4<T> o;
@@ -98,13 +96,6 @@ template <typename T, bool JAC> struct ProCgDir {
     prefetch_l2(r + i, cnt * sizeof(T));
     if (JAC) prefetch_l2(D + i, cnt * sizeof(T));
     if (beta != (T)0) prefetch_l2(p + i, cnt * sizeof(T));
-  }
-  __device__ T operator()(size_t i) const {
-    const T ri = __ldg(r + i);
-    const T zi = JAC ? jprec(ri, __ldg(D + i), c) : ri;
-    const T pn = beta == (T)0 ? zi : zi + beta * __ldg(p + i);
-    p[i] = pn;
-    return pn;
   }
   __device__ V4<T> vec4(size_t i) const {
     const V4<T> rv = ld4(r + i);

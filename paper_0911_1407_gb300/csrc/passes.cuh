@@ -127,34 +127,29 @@ k_xf(Pro pro, cpx<T>* __restrict__ A, FftPlan plan, const cpx<T>* __restrict__ t
   const int z = blockIdx.y, y0 = blockIdx.x * G::RY;
   const int rows = min(G::RY, n - y0);
   const int lines = rows >> 1;
-  if (n & 3) {   // rows not a multiple of 4 long: one element per step
-    for (int e = threadIdx.x; e < rows * n; e += kThreads) {
-      const int row = fdiv(e, plan.nd), x = e - row * n;
-      reinterpret_cast<T*>(&a[x * G::P + (row >> 1)])[row & 1] =
-          pro(((size_t)z * n + (y0 + row)) * n + x);
-    }
-  }
-  // four consecutive x per thread and step: 16-byte global accesses
-  const int total4 = (n & 3) ? 0 : (rows * n) >> 2;
+  // four consecutive elements of the tile per thread and step: the tile's rows
+  // are contiguous and n, rows and y0 even, so 16-byte accesses hold for any n
+  // (where n is not a multiple of 4, a step may end in the next row)
+  const int total4 = (rows * n) >> 2;
+  const size_t row0 = ((size_t)z * n + y0) * n;
   constexpr int B = 4;
   for (int base = threadIdx.x; base < total4; base += B * kThreads) {
     V4<T> u[B];
 #pragma unroll
     for (int k = 0; k < B; ++k) {
       const int e = base + k * kThreads;
-      if (e < total4) {
-        const int row = fdiv(4 * e, plan.nd), x = 4 * e - row * n;
-        u[k] = pro.vec4(((size_t)z * n + (y0 + row)) * n + x);
-      }
+      if (e < total4) u[k] = pro.vec4(row0 + 4 * (size_t)e);
     }
 #pragma unroll
     for (int k = 0; k < B; ++k) {
       const int e = base + k * kThreads;
       if (e < total4) {
-        const int row = fdiv(4 * e, plan.nd), x = 4 * e - row * n;
+        int row = fdiv(4 * e, plan.nd), x = 4 * e - row * n;
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          reinterpret_cast<T*>(&a[(x + j) * G::P + (row >> 1)])[row & 1] = u[k].v[j];
+        for (int j = 0; j < 4; ++j) {
+          reinterpret_cast<T*>(&a[x * G::P + (row >> 1)])[row & 1] = u[k].v[j];
+          if (++x == n) { x = 0; ++row; }
+        }
       }
     }
   }
@@ -261,6 +256,52 @@ k_yi(const cpx<T>* __restrict__ B, cpx<T>* __restrict__ A, FftPlan plan,
 }
 
 // ---------------------------------------------------------------------------
+// YZY: the YF, Z and YI passes of a whole kx plane in one block, in place on
+// A[:][kx][:], for planes of which two fit in shared memory (the Stockham
+// stages ping-pong).  grid = n/2+1.  The same operations on the same values as
+// the three passes.
+// ---------------------------------------------------------------------------
+constexpr int kPlaneThreads = 512;
+template <typename T> inline size_t plane_smem(int n) {
+  return sizeof(cpx<T>) * ((size_t)n + 2 * (size_t)n * (n + 1));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kPlaneThreads)
+k_yzy(cpx<T>* __restrict__ A, const T* __restrict__ M, int zero_dc, FftPlan plan,
+      const cpx<T>* __restrict__ twg, const int* __restrict__ done) {
+  using C = cpx<T>;
+  if (done && *done) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n = plan.n, h = n / 2 + 1, S = n + 1, kx = blockIdx.x;
+  C* tw = reinterpret_cast<C*>(smem_raw);
+  C *a = tw + n, *b = a + n * S;
+  C* const plane = A + (size_t)kx * n;
+  load_twiddles<T>(tw, twg, n);
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+    const int z = fdiv(e, plan.nd), y = e - z * n;
+    cp_async(&a[z * S + y], &plane[(size_t)z * h * n + y]);
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  fft_lines_n<T, -1>(a, b, plan, n, S, 1, tw);      // lines z along y
+  fft_lines_n<T, -1>(a, b, plan, n, 1, S, tw);      // lines ky along z
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+    const int kz = fdiv(e, plan.nd), ky = e - kz * n;
+    const int my = min(ky, n - ky), mz = min(kz, n - kz);
+    const int m2 = kx * kx + my * my + mz * mz;
+    a[kz * S + ky] = cscale(a[kz * S + ky], (zero_dc && m2 == 0) ? (T)0 : __ldg(M + m2));
+  }
+  __syncthreads();
+  fft_lines_n<T, +1>(a, b, plan, n, 1, S, tw);
+  fft_lines_n<T, +1>(a, b, plan, n, S, 1, tw);
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+    const int z = fdiv(e, plan.nd), y = e - z * n;
+    plane[(size_t)z * h * n + y] = a[z * S + y];
+  }
+}
+
+// ---------------------------------------------------------------------------
 // XI: c2r along x + epilogue.  grid = (ceil(n / RY), n).  Rows 2j and 2j+1
 // are recovered together from Z[k] = X_a[k] + i X_b[k] (k <= n/2) and
 // Z[n-k] = conj X_a[k] + i conj X_b[k]; the imaginary parts of the k = 0 and
@@ -309,6 +350,7 @@ k_xi(const cpx<T>* __restrict__ A, Epi epi, Fin fin, RedArgs ra, FftPlan plan,
 #pragma unroll
   for (int j = 0; j < Epi::NV; ++j) acc[j].init((Epi::MAXMASK >> j) & 1u);
   if (n & 3) {   // rows not a multiple of 4 long: one element per step
+#pragma unroll 4
     for (int e = threadIdx.x; e < rows * n; e += kThreads) {
       const int row = fdiv(e, plan.nd), x = e - row * n;
       const C zz = a[x * G::P + (row >> 1)];

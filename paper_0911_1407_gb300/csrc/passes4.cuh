@@ -293,6 +293,128 @@ k4_yi(const cpx<T>* __restrict__ B, cpx<T>* __restrict__ A, const cpx<T>* __rest
   }
 }
 
+// ---------------------------------------------------------------------------
+// YZY: the y-forward, z and y-inverse passes of a whole kx plane in one block,
+// for planes that fit in shared memory (n <= 128).  grid = n/2+1; block kx
+// reads and writes A[:][kx][:] in place.  P[z][y], pitch N + 1, holds the
+// plane; every phase rewrites the slots it read, so a barrier between phases
+// is all they need: ky sits at slot (ky % N1) N2 + ky / N1 of its row between
+// the y transforms, kz at row (kz % N1) N2 + kz / N1 between the z transforms'
+// phases.  The same operations on the same values as the three passes, so the
+// same bits; what goes is four trips of the spectrum through L2 and two
+// launches.
+// ---------------------------------------------------------------------------
+template <int N1, int N2> struct GeoP {
+  static constexpr int N = N1 * N2, S = N + 1;
+  // tasks of a phase are N N2 or N N1; a thread's share of them is unrolled
+  static constexpr int kT = N >= 64 ? 512 : 256;
+  template <typename C> static constexpr size_t smem() { return sizeof(C) * (N + (size_t)N * S); }
+};
+
+template <typename T, int N1, int N2>
+__global__ void __launch_bounds__(GeoP<N1, N2>::kT)
+k4_yzy(cpx<T>* __restrict__ A, const T* __restrict__ M, int zero_dc,
+       const cpx<T>* __restrict__ twg, const int* __restrict__ done) {
+  using Gm = GeoP<N1, N2>;
+  using C = cpx<T>;
+  constexpr int N = Gm::N, S = Gm::S, kT = Gm::kT;
+  if (done && *done) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* tw2 = reinterpret_cast<C*>(smem_raw);
+  C* P = tw2 + N;
+  const int h = N / 2 + 1, kx = blockIdx.x;
+  C* const plane = A + (size_t)kx * N;
+  load_tw2<C, N1, N2>(tw2, twg);
+  __syncthreads();
+  // tasks (line, n2) with n2 on consecutive lanes, (line, k1) and the column
+  // tasks with the line on consecutive lanes
+  for (int t = threadIdx.x; t < N * N2; t += kT) {
+    const int z = t / N2, n2 = t % N2;
+    const C* src = plane + (size_t)z * h * N + n2;
+    C v[N1];
+#pragma unroll
+    for (int n1 = 0; n1 < N1; ++n1) v[n1] = src[N2 * n1];
+    phase_a<T, N1, N2, -1>(v, tw2, n2);
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) P[z * S + k1 * N2 + n2] = v[k1];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < N * N1; t += kT) {
+    C* q = P + (t % N) * S + (t / N) * N2;
+    C v[N2];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) v[n2] = q[n2];
+    dft_small<T, -1, N2>(v);
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) q[k2] = v[k2];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < N * N2; t += kT) {
+    const int c = t % N, n2 = t / N;
+    C* q = P + n2 * S + c;
+    C v[N1];
+#pragma unroll
+    for (int n1 = 0; n1 < N1; ++n1) v[n1] = q[N2 * n1 * S];
+    phase_a<T, N1, N2, -1>(v, tw2, n2);
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) q[N2 * k1 * S] = v[k1];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < N * N1; t += kT) {
+    const int c = t % N, k1 = t / N;
+    const int ky = c / N2 + N1 * (c % N2), my = min(ky, N - ky), m1 = kx * kx + my * my;
+    C* q = P + k1 * N2 * S + c;
+    T mult[N2];
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) {
+      const int kz = k1 + N1 * k2, mz = min(kz, N - kz), m2 = m1 + mz * mz;
+      mult[k2] = zero_dc && m2 == 0 ? T(0) : __ldg(M + m2);
+    }
+    C v[N2];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) v[n2] = q[n2 * S];
+    dft_small<T, -1, N2>(v);
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) v[k2] = cscale(v[k2], mult[k2]);
+    phase_b_inv<T, N1, N2>(v, tw2, k1);
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) q[n2 * S] = v[n2];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < N * N2; t += kT) {
+    const int c = t % N, n2 = t / N;
+    C* q = P + n2 * S + c;
+    C v[N1];
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) v[k1] = q[N2 * k1 * S];
+    dft_small<T, +1, N1>(v);
+#pragma unroll
+    for (int n1 = 0; n1 < N1; ++n1) q[N2 * n1 * S] = v[n1];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < N * N1; t += kT) {
+    const int k1 = t / N;
+    C* q = P + (t % N) * S + k1 * N2;
+    C v[N2];
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) v[k2] = q[k2];
+    phase_b_inv<T, N1, N2>(v, tw2, k1);
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) q[n2] = v[n2];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < N * N2; t += kT) {
+    const int z = t / N2, n2 = t % N2;
+    C v[N1];
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) v[k1] = P[z * S + k1 * N2 + n2];
+    dft_small<T, +1, N1>(v);
+    C* dst = plane + (size_t)z * h * N + n2;
+#pragma unroll
+    for (int n1 = 0; n1 < N1; ++n1) dst[N2 * n1] = v[n1];
+  }
+}
+
 // Frequencies of the paired x-pass tasks: warp g < N1/2 takes k1 = g and
 // N1 - g on its two half-warps (g = 0: k1 = 0 and N1/2, each its own partner).
 template <int N1> __device__ __forceinline__ int pair_k1(int g, int member) {
