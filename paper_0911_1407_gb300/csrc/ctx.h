@@ -9,6 +9,7 @@
 
 #include "../../include/plc.h"
 #include "common.cuh"
+#include "ctl.cuh"
 
 namespace plc {
 
@@ -166,7 +167,8 @@ template <typename T, typename TC>
 void newton_update(plc_ctx* c, const T* s, const T* y, const T* g, const TC* r, const TC* xi,
                    const TC* D, const int32_t* N, const double* w, double nbar, double tau,
                    bool jac, T* s2, T* y2, T* g2, TC* D2, TC* r2,
-                   const double* tau_dev = nullptr);   // non-null: tau read on the device
+                   const double* tau_dev = nullptr,    // non-null: tau read on the device
+                   const LoopCtl& loop = LoopCtl{});
 template <typename T> void cg_hv(plc_ctx* c, const T* r, const T* D, T* p, T* Hp, bool jac);
 // The Gaussian-prior model (Eq. MAPG): gradient through the FFT at delta,
 // line-search trial, and the fraction-to-boundary quantity (into sc->bmax).
@@ -191,7 +193,8 @@ template <typename TC> void lsq_init(plc_ctx* c, const int32_t* N, const double*
 template <typename TC> void precond(plc_ctx* c, const TC* D, const TC* r, bool jac);
 // rtol2 < 0: the stopping parameters are read from the device scalars.
 template <typename TC> void cg_update(plc_ctx* c, TC* x, TC* r, const TC* p, const TC* Hp,
-                                      const TC* D, bool jac, double rtol2, int max_iter);
+                                      const TC* D, bool jac, double rtol2, int max_iter,
+                                      const LoopCtl& loop = LoopCtl{});
 template <typename TC> void diag(plc_ctx* c, const double* s, const double* w, double nbar, TC* D);
 template <typename TD, typename TS> void convert(plc_ctx* c, const TS* src, TD* dst);
 // Start point of the lognormal solve: the MAP of the same posterior with the

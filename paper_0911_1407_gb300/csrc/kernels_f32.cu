@@ -14,7 +14,8 @@ template void grad_newton<float, float, float>(plc_ctx*, const float*, const dou
 template void newton_update<float, float>(plc_ctx*, const float*, const float*, const float*,
                                           const float*, const float*, const float*,
                                           const int32_t*, const double*, double, double, bool,
-                                          float*, float*, float*, float*, float*, const double*);
+                                          float*, float*, float*, float*, float*, const double*,
+                                            const LoopCtl&);
 template void grad_newton_g<float, float, float>(plc_ctx*, const float*, const double*,
                                                  const int32_t*, double, float*, float*, float*,
                                                  float*, bool);
@@ -31,7 +32,7 @@ template void lsq_init<float>(plc_ctx*, const int32_t*, const double*, double, f
                               bool);
 template void cg_init<float>(plc_ctx*, const double*, const float*, float*, bool);
 template void cg_update<float>(plc_ctx*, float*, float*, const float*, const float*, const float*,
-                               bool, double, int);
+                               bool, double, int, const LoopCtl&);
 template void diag<float>(plc_ctx*, const double*, const double*, double, float*);
 template void convert<double, float>(plc_ctx*, const float*, double*);
 template void convert<float, double>(plc_ctx*, const double*, float*);

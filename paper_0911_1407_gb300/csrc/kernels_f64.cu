@@ -22,17 +22,19 @@ template void newton_update<double, double>(plc_ctx*, const double*, const doubl
                                             const double*, const double*, const double*,
                                             const int32_t*, const double*, double, double, bool,
                                             double*, double*, double*, double*, double*,
-                                            const double*);
+                                            const double*,
+                                            const LoopCtl&);
 template void newton_update<double, float>(plc_ctx*, const double*, const double*, const double*,
                                            const float*, const float*, const float*,
                                            const int32_t*, const double*, double, double, bool,
                                            double*, double*, double*, float*, float*,
-                                           const double*);
+                                           const double*,
+                                            const LoopCtl&);
 template void cg_hv<double>(plc_ctx*, const double*, const double*, double*, double*, bool);
 template void diag_start<double>(plc_ctx*, double*, const int32_t*, const double*, double);
 template void cg_init<double>(plc_ctx*, const double*, const double*, double*, bool);
 template void cg_update<double>(plc_ctx*, double*, double*, const double*, const double*,
-                                const double*, bool, double, int);
+                                const double*, bool, double, int, const LoopCtl&);
 template void diag<double>(plc_ctx*, const double*, const double*, double, double*);
 template void precond<double>(plc_ctx*, const double*, const double*, bool);
 }  // namespace plc

@@ -376,7 +376,8 @@ template <typename TC> void precond(plc_ctx* c, const TC* D, const TC* r, bool j
 }
 
 template <typename TC> void cg_update(plc_ctx* c, TC* x, TC* r, const TC* p, const TC* Hp,
-                                      const TC* D, bool jac, double rtol2, int max_iter) {
+                                      const TC* D, bool jac, double rtol2, int max_iter,
+                                      const LoopCtl& loop) {
   // one wave (FP32: 4 blocks of 256 per SM at its 56 registers, 73.8 us
   // against 77.1 with two waves at 256^3)
     const int nb = pointwise_blocks((long long)c->n3(), c->sms, sizeof(TC) == 8 ? 3 : 4);
@@ -384,23 +385,24 @@ template <typename TC> void cg_update(plc_ctx* c, TC* x, TC* r, const TC* p, con
   if (jac)
     k_cg_update<TC, true><<<nb, kThreads, 0, c->stream>>>(x, r, p, Hp, precond_field<TC>(c, D),
                                                            (TC)c->jac_c, c->n3(), red_args(c),
-                                                           rtol2, max_iter);
+                                                           rtol2, max_iter, loop);
   else
     k_cg_update<TC, false><<<nb, kThreads, 0, c->stream>>>(x, r, p, Hp, D, (TC)c->jac_c, c->n3(),
-                                                            red_args(c), rtol2, max_iter);
+                                                            red_args(c), rtol2, max_iter, loop);
   check(cudaGetLastError(), "k_cg_update");
 }
 
 template <typename T, typename TC>
 void newton_update(plc_ctx* c, const T* s, const T* y, const T* g, const TC* r, const TC* xi,
                    const TC* D, const int32_t* N, const double* w, double nbar, double tau,
-                   bool jac, T* s2, T* y2, T* g2, TC* D2, TC* r2, const double* tau_dev) {
+                   bool jac, T* s2, T* y2, T* g2, TC* D2, TC* r2, const double* tau_dev,
+                   const LoopCtl& loop) {
   // g may be left out only where forming it again from y, D and N is exact
   if (!g && !std::is_same<T, TC>::value) check(cudaErrorInvalidValue, "newton_update without g");
   LaunchScope ls(c, sizeof(T) == 4 ? S_NEWTON_UPDATE32 : S_NEWTON_UPDATE64);
   k_newton_update<T, TC><<<pw_blocks(c), kThreads, 0, c->stream>>>(
       s, y, g, r, xi, D, N, w, nbar, c->mu, tau, tau_dev, c->jac_c, jac ? 1 : 0, s2, y2, g2, D2, r2,
-      c->n3(), red_args(c));
+      c->n3(), red_args(c), loop);
   check(cudaGetLastError(), "k_newton_update");
 }
 

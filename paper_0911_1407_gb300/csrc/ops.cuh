@@ -12,6 +12,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "ctl.cuh"
 #include "log64.cuh"
 #include "ff.cuh"
 
@@ -592,8 +593,12 @@ template <typename TC, bool JAC>
 __global__ void __launch_bounds__(kThreads, sizeof(TC) == 8 ? 3 : 1)
 k_cg_update(TC* __restrict__ x, TC* __restrict__ r, const TC* __restrict__ p,
             const TC* __restrict__ Hp, const TC* __restrict__ D, TC c, size_t n3,
-            RedArgs ra, double rtol2, int max_iter) {
-  if (ra.sc->done) return;
+            RedArgs ra, double rtol2, int max_iter, LoopCtl loop) {
+  if (ra.sc->done) {
+    // a breakdown in the product: nothing to update, but the loop must end
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl_cg(loop, 1);
+    return;
+  }
   const TC alpha = (TC)ra.sc->alpha;
   const bool first = ra.sc->iter == 0;
   typename AccOf<TC>::type a0, a1, a2;
@@ -624,6 +629,7 @@ k_cg_update(TC* __restrict__ x, TC* __restrict__ r, const TC* __restrict__ p,
   struct Fin {
     double rtol2;
     int max_iter;
+    LoopCtl loop;
     __device__ void operator()(const double* t, DevScalars* sc) const {
       const double rt2 = rtol2 < 0.0 ? sc->rtol2 : rtol2;
       const int mi = rtol2 < 0.0 ? sc->max_iter : max_iter;
@@ -632,10 +638,12 @@ k_cg_update(TC* __restrict__ x, TC* __restrict__ r, const TC* __restrict__ p,
       sc->rr = t[1];
       sc->xmax = t[2];
       sc->iter += 1;
-      if (t[1] <= rt2 * sc->bnorm2 || sc->iter >= mi) sc->done = 1;
+      const int end = t[1] <= rt2 * sc->bnorm2 || sc->iter >= mi;
+      if (end) sc->done = 1;
+      ctl_cg(loop, end);
     }
   };
-  block_reduce_finish_acc<3, 1u << 2>(acc, ra, Fin{rtol2, max_iter});
+  block_reduce_finish_acc<3, 1u << 2>(acc, ra, Fin{rtol2, max_iter, loop});
 }
 
 // A Newton trial point without an FFT.  S^-1 is linear, so with the CG's
@@ -658,7 +666,7 @@ k_newton_update(const T* __restrict__ s, const T* __restrict__ y, const T* __res
                 double mu, double tau_arg, const double* __restrict__ tau_dev, double c,
                 int jac, T* __restrict__ s2,
                 T* __restrict__ y2, T* __restrict__ g2, TC* __restrict__ D2,
-                TC* __restrict__ r2, size_t n3, RedArgs ra) {
+                TC* __restrict__ r2, size_t n3, RedArgs ra, LoopCtl loop) {
   using Acc = typename AccOf<T>::type;
   constexpr int NS = sizeof(TC) == 8 ? 5 : 6;   // k_precond takes the last sum (FP64 CG)
   Acc acc[NS];
@@ -710,7 +718,14 @@ k_newton_update(const T* __restrict__ s, const T* __restrict__ y, const T* __res
     st4(D2 + i, dout);
     st4(r2 + i, rout);
   }
-  block_reduce_finish_acc<NS, 0u>(acc, ra, FinGrad<NS>{});
+  struct Fin {
+    LoopCtl loop;
+    __device__ void operator()(const double* t, DevScalars* sc) const {
+      FinGrad<NS>{}(t, sc);
+      ctl_ls(loop, sc);
+    }
+  };
+  block_reduce_finish_acc<NS, 0u>(acc, ra, Fin{loop});
 }
 
 // D = nbar w e^s (Sec. 3.1.2), from an FP64 s.

@@ -57,20 +57,24 @@ __global__ void k_build_bias(double* __restrict__ M64, float* __restrict__ M32, 
 
 // (S^-1)_ii = n^-3 sum_k 1/lambda_k = sum over all n^3 modes of M[|m|^2],
 // and the prior variance per cell without the DC mode,
-// S_ii = n^-3 sum_{k != 0} lambda_k = n^-6 sum_{k != 0} 1 / M[|m|^2].
+// S_ii = n^-3 sum_{k != 0} lambda_k = n^-6 sum_{k != 0} 1 / M[|m|^2].  Over the
+// octant 0 <= m <= n/2 with each component's multiplicity (1 at 0 and n/2,
+// else 2): a table value and an FP64 quotient per mode, 92 us at 128^3 over
+// all modes.
 __global__ void __launch_bounds__(kThreads)
 k_jacobi_constant(const double* __restrict__ M64, int n, RedArgs ra) {
   double acc[2] = {0.0, 0.0};
-  const size_t n3 = (size_t)n * n * n;
+  const int h = n / 2 + 1, nh = n / 2;
+  const size_t n3 = (size_t)n * n * n, oct = (size_t)h * h * h;
   const double inv_n6 = 1.0 / ((double)n3 * (double)n3);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n3;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < oct;
        i += (size_t)gridDim.x * blockDim.x) {
-    const int kx = (int)(i % n), ky = (int)((i / n) % n), kz = (int)(i / ((size_t)n * n));
-    const int mx = min(kx, n - kx), my = min(ky, n - ky), mz = min(kz, n - kz);
+    const int mx = (int)(i % h), my = (int)((i / h) % h), mz = (int)(i / ((size_t)h * h));
     const int m2 = mx * mx + my * my + mz * mz;
-    const double v = M64[m2];
-    acc[0] += v;
-    if (m2 > 0 && v > 0.0) acc[1] += inv_n6 / v;
+    auto twice = [&](int m) { return m == 0 || m == nh ? 1 : 2; };
+    const double v = M64[m2], mult = (double)(twice(mx) * twice(my) * twice(mz));
+    acc[0] += mult * v;
+    if (m2 > 0 && v > 0.0) acc[1] += mult * (inv_n6 / v);
   }
   block_reduce_finish<2, 0u>(acc, ra, FinStore<2>{});
 }
