@@ -1,16 +1,15 @@
 // ff.cuh -- float-float ("double-word") arithmetic on the FP32 pipes.
 //
 // A real is held as the unevaluated sum hi + lo of two floats with
-// |lo| <= ulp(hi) / 2: about 48 significant bits, for transforms that need
-// more than FP32 at a fraction of the cost of GB300's FP64 rate (1/64 of
+// |lo| <= ulp(hi) / 2: about 48 significant bits, for the epilogue of the mixed
+// solve's FP64 gradient at a fraction of the cost of GB300's FP64 rate (1/64 of
 // FP32).  Built from the error-free transforms TwoSum (Knuth, The Art of
 // Computer Programming vol. 2, Sec. 4.2.2), Fast2Sum (Dekker, Numer. Math.
 // 18, 1971) and the exact product by FMA (a*b - fl(a*b) = fma(a, b,
 // -fl(a*b))), as analysed for double-word numbers by Joldes, Muller &
 // Popescu (ACM TOMS 44, 2017):
 //   - sum: the high parts added exactly, the low parts added to the error
-//     term, one renormalisation (the error is a few 2^-48 of |a| + |b|,
-//     which is what the butterflies of an FFT need);
+//     term, one renormalisation (the error is a few 2^-48 of |a| + |b|);
 //   - product: exact product of the high parts, the cross terms added by
 //     FMA, one renormalisation.
 // The compiler must not reassociate these expressions (nvcc does not without
