@@ -245,8 +245,7 @@ plc_status plc_create(plc_ctx** out, int n, double box, int precision, void* str
       // long double has at least 64 significant bits on the hosts in use
       const long double al = 2.0L * std::acos(-1.0L) * (long double)m / (long double)n;
       const long double one = (long double)(1ll << plc::kFxOne);
-      tfx[m] = plc::fxw{plc::fx_split(std::llrint(std::cos(al) * one)),
-                        plc::fx_split(std::llrint(-std::sin(al) * one))};
+      tfx[m] = plc::fx_factor(std::llrint(std::cos(al) * one), std::llrint(-std::sin(al) * one));
       t32[m] = make_float2((float)t64[m].x, (float)t64[m].y);
     }
     plc::check(cudaMemcpyAsync(c->tw64, t64.data(), sizeof(double2) * n, cudaMemcpyHostToDevice, c->stream), "copy twiddles");

@@ -22,7 +22,7 @@
 // What bounds them: the FP64 Stockham passes they replace ran at 0.74-0.8 of
 // the FP64 pipe (2 per SM and clock).  These issue on half of all cycles with
 // 16 warps per SM (128 registers), the integer adders 45-60% busy.  S^-1 at
-// 128^3 / 192^3 / 256^3 went from 327 / 1170 / 3450 us to 88 / 263 / 480.
+// 128^3 / 192^3 / 256^3 went from 327 / 1170 / 3450 us to 88 / 264 / 470.
 #pragma once
 
 #include "ctx.h"
@@ -57,6 +57,11 @@ template <int N1_, int N2_> struct GeoX : Geo4<fx, N1_, N2_> {
   static_assert(fixed_length(N1_ * N2_), "listed as a fixed-point length");
   using G = Geo4<fx, N1_, N2_>;
   static constexpr int NM = N1_ > N2_ ? N1_ : N2_;
+  static constexpr size_t tw_bytes = sizeof(fxw) * N1_ * N2_;
+  static constexpr size_t smem_y = tw_bytes + G::x_bytes;
+  static constexpr size_t smem_z = smem_y + G::m_bytes;
+  static constexpr size_t smem_x = tw_bytes + (G::x_bytes > G::r_bytes ? G::x_bytes : G::r_bytes);
+  static_assert(tw_bytes % 16 == 0, "the exchange buffer follows the twiddles");
   // per-thread L1 parts: line c at [c * (NM + 1)]
   static constexpr int red_words = G::L * (NM + 1) + 8;
 };
@@ -71,13 +76,13 @@ template <int N1, int N2, int SIGN>
 __device__ __forceinline__ void phase_a_x(fxc* v, const fxw* tw, int n2) {
   dft_small<fx, SIGN, N1>(v);
 #pragma unroll
-  for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmul(v[k1], conj_if<SIGN>(tw[k1 * N2 + n2]));
+  for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmulx<SIGN>(v[k1], tw[k1 * N2 + n2]);
 }
 template <int N1, int N2>
 __device__ __forceinline__ void phase_b_inv_x(fxc* v, const fxw* tw, int k1) {
   dft_small<fx, +1, N2>(v);
 #pragma unroll
-  for (int n2 = 1; n2 < N2; ++n2) v[n2] = cmul(v[n2], conj_if<+1>(tw[k1 * N2 + n2]));
+  for (int n2 = 1; n2 < N2; ++n2) v[n2] = cmulx<+1>(v[n2], tw[k1 * N2 + n2]);
 }
 
 // The largest L1 norm over the block's 16 lines from the parts of the tasks
