@@ -185,11 +185,13 @@ __device__ __forceinline__ float exp2_le0(int d) {
 __device__ __forceinline__ float fx_mag(fx a) { return fabsf((float)(int)(a.v >> 32)); }
 __device__ __forceinline__ float fx_mag(fxc a) { return fx_mag(a.x) + fx_mag(a.y); }
 
-// q 2^-s rounded to nearest, s >= 0 (half = 2^(s-1), 0 for s = 0).
+// q 2^-s rounded to nearest, s >= 0 (half = 2^(s-1), 0 for s = 0).  |q| <= 2^62,
+// so every shift from 63 on gives 0.
 struct FxShift {
   int s;
   long long half;
-  __device__ __forceinline__ explicit FxShift(int d) : s(min(max(d, 0), 63)), half((1ll << s) >> 1) {}
+  __device__ __forceinline__ explicit FxShift(int d)
+      : s(min(max(d, 0), 63)), half((long long)((1ull << s) >> 1)) {}
   __device__ __forceinline__ fx operator()(fx a) const { return fx{(a.v + half) >> s}; }
   __device__ __forceinline__ fxc operator()(fxc a) const { return fxc{(*this)(a.x), (*this)(a.y)}; }
 };

@@ -1,0 +1,61 @@
+"""Values far below the quantum of the fixed-point FP64 passes: they count as
+nothing, not as one quantum of a fixed sign.
+
+The fields are chosen so that the passes are exact, or round once in a place
+that can be named, where one quantum too many in each of a line's elements
+shows.
+"""
+import pytest
+import torch
+
+from tests.gpu_util import ensure_lib, pk_table_for
+
+pytestmark = pytest.mark.gpu
+
+SIDES = [32, 64, 96, 128, 192, 256]
+
+
+@pytest.fixture(scope="module")
+def plc():
+    return ensure_lib()
+
+
+def _context(plc, n):
+    c = plc.Context(n, 5.0 * n, "fp64")
+    k, P = pk_table_for(n, 5.0 * n, seed=n)
+    c.set_prior(k, P, -0.2)
+    return c
+
+
+# (the inverse of 192 = 16 x 12 takes this wave through a radix 3, which rounds)
+@pytest.mark.parametrize("n", [n for n in SIDES if n != 192])
+def test_zero_planes_add_nothing(plc, n):
+    # (-1)^y on the plane z = 0, zero elsewhere: only the modes (0, n/2, kz)
+    # are not zero, so the result is v(z) (-1)^y.  All-zero lines lie beside
+    # the one that is not in the tiles of every pass.  Past the inverse y
+    # transform, which gives +-v exactly, v and -v are shifted once (a tie
+    # rounds up: they part by at most one quantum, which is below 2^-59 of the
+    # largest v of the 16 planes that share an exponent; twice that allowed)
+    # and rounded to double (half an ulp each).
+    c = _context(plc, n)
+    sign = 1.0 - 2.0 * (torch.arange(n, device="cuda", dtype=torch.float64) % 2)
+    x = torch.zeros((n, n, n), dtype=torch.float64, device="cuda")
+    x[0] = sign[:, None]
+    y = c.prior_apply(x)
+    v = y[:, 0, 0].abs()
+    top = v.view(-1, 16).amax(1).repeat_interleave(16)
+    off = (y - y[:, :1, :1] * sign[None, :, None]).abs().amax((1, 2))
+    assert bool((v > 0).any())
+    assert bool((off <= 2.0 ** -58 * top + 2.0 ** -52 * v).all())
+
+
+@pytest.mark.parametrize("n", SIDES)
+def test_vanishing_multipliers_add_nothing(plc, n):
+    # a constant plus a wave of y at the highest frequency, smoothed by a
+    # Gaussian that leaves nothing of the wave: a constant, to the last bit
+    c = _context(plc, n)
+    sign = 1.0 - 2.0 * (torch.arange(n, device="cuda", dtype=torch.float64) % 2)
+    x = (1.5 + sign)[None, :, None].expand(n, n, n).contiguous()
+    y = c.smooth(x, 5.0 * n)
+    assert torch.equal(y, torch.full_like(y, float(y[0, 0, 0])))
+    assert abs(float(y[0, 0, 0]) - 1.5) <= 1e-15
