@@ -196,13 +196,14 @@ struct FxShift {
   __device__ __forceinline__ fxc operator()(fxc a) const { return fxc{(*this)(a.x), (*this)(a.y)}; }
 };
 
-// double -> quanta of 2^E, where |d| < 2^(E + 62); zero and subnormal d give 0.
+// double -> quanta of 2^E, rounded to nearest, where |d| < 2^(E + 62); zero and
+// subnormal d give 0.
 __device__ __forceinline__ fx fx_from(double d, int E) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(d);
   const int ex = (int)(b >> 52) & 0x7ff;
   const unsigned long long m = (((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 10);
-  const int s = min(max(E - ex + 1085, 1), 63);
-  const long long q = ex == 0 ? 0ll : (long long)((m + (1ull << (s - 1))) >> s);
+  const int sh = E - ex + 1085, s = min(max(sh, 1), 63);
+  const long long q = ex == 0 || sh > 63 ? 0ll : (long long)((m + (1ull << (s - 1))) >> s);
   const long long sg = (long long)b >> 63;
   return fx{(q ^ sg) - sg};
 }

@@ -59,3 +59,15 @@ def test_vanishing_multipliers_add_nothing(plc, n):
     y = c.smooth(x, 5.0 * n)
     assert torch.equal(y, torch.full_like(y, float(y[0, 0, 0])))
     assert abs(float(y[0, 0, 0]) - 1.5) <= 1e-15
+
+
+@pytest.mark.parametrize("n", SIDES)
+def test_a_background_below_the_quantum_adds_nothing(plc, n):
+    # 1e-300 beside 1 is nothing in double as in the passes: the same bits
+    c = _context(plc, n)
+    x = torch.zeros((n, n, n), dtype=torch.float64, device="cuda")
+    x[n // 2, 1, n - 1] = 1.0
+    y = c.prior_apply(x)
+    for tiny in (1e-300, -1e-300, 1e-30):
+        b = torch.where(x == 0.0, torch.full_like(x, tiny), x)
+        assert torch.equal(c.prior_apply(b), y)
