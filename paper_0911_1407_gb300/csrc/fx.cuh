@@ -170,7 +170,7 @@ template <int SIGN> struct Dft<fx, SIGN> {
 
 // ------------------------------ tile exponents ------------------------------
 constexpr int kFxNaN = 1 << 20;      // tile holds a NaN or an infinity
-constexpr int kFxNone = -(1 << 20);  // tile is all zeros
+constexpr int kFxNone = -(1 << 20);  // below the exponent of any tile
 constexpr int kFxBits = 62;          // L1 of a line stays below 2^62 quanta
 
 // Smallest b with l1 (1 + 2^-10) < 2^b (l1 > 0).
@@ -196,14 +196,14 @@ struct FxShift {
   __device__ __forceinline__ fxc operator()(fxc a) const { return fxc{(*this)(a.x), (*this)(a.y)}; }
 };
 
-// double -> quanta of 2^E, rounded to nearest, where |d| < 2^(E + 62); zero and
-// subnormal d give 0.
+// double -> quanta of 2^E, rounded to nearest, where |d| < 2^(E + 62) and, for
+// subnormal d, E >= -1083.
 __device__ __forceinline__ fx fx_from(double d, int E) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(d);
-  const int ex = (int)(b >> 52) & 0x7ff;
-  const unsigned long long m = (((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 10);
-  const int sh = E - ex + 1085, s = min(max(sh, 1), 63);
-  const long long q = ex == 0 || sh > 63 ? 0ll : (long long)((m + (1ull << (s - 1))) >> s);
+  const int ex = (int)(b >> 52) & 0x7ff;   // 0 (zero, subnormal): no implicit bit
+  const unsigned long long m = (((b & 0xFFFFFFFFFFFFFull) | (ex ? 1ull << 52 : 0ull)) << 10);
+  const int sh = E - max(ex, 1) + 1085, s = min(max(sh, 1), 63);
+  const long long q = sh > 63 ? 0ll : (long long)((m + (1ull << (s - 1))) >> s);
   const long long sg = (long long)b >> 63;
   return fx{(q ^ sg) - sg};
 }

@@ -173,11 +173,21 @@ kx_xf(Pro pro, fxc* __restrict__ A, FxExps ex, const fxw* __restrict__ twg,
     auto mag = [&](double x) {
       return __uint_as_float((unsigned)max((__double2hiint(x) & 0x7fffffff) - off, 0) << 3);
     };
+    if (exm != 0) {
 #pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) part += mag(ra[N2 * n1]) + mag(rb[N2 * n1]);
+      for (int n1 = 0; n1 < N1; ++n1) part += mag(ra[N2 * n1]) + mag(rb[N2 * n1]);
+    } else {   // zeros and subnormals, in units of 2^-1042
+#pragma unroll 1
+      for (int n1 = 0; n1 < N1; ++n1)
+        part += (float)((__double2hiint(ra[N2 * n1]) & 0x7fffffff) +
+                        (__double2hiint(rb[N2 * n1]) & 0x7fffffff) + 2);
+    }
   }
   const float l1 = block_l1<N2, Gm::NM>(red, task_a, ca, n2a, part);
-  const int E = exm == 2047 ? kFxNaN : (exm == 0 ? kFxNone : exm - 1023 + l1_bits(l1) - kFxBits);
+  // (-1083: the finest quantum fx_from converts subnormals to)
+  const int E = exm == 2047 ? kFxNaN
+                : exm == 0  ? max(-1042 + l1_bits(l1) - kFxBits, -1083)
+                            : exm - 1023 + l1_bits(l1) - kFxBits;
   C v[Gm::NM];
   if (task_a) {
 #pragma unroll

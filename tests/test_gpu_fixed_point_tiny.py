@@ -5,6 +5,7 @@ The fields are chosen so that the passes are exact, or round once in a place
 that can be named, where one quantum too many in each of a line's elements
 shows.
 """
+import numpy as np
 import pytest
 import torch
 
@@ -71,3 +72,19 @@ def test_a_background_below_the_quantum_adds_nothing(plc, n):
     for tiny in (1e-300, -1e-300, 1e-30):
         b = torch.where(x == 0.0, torch.full_like(x, tiny), x)
         assert torch.equal(c.prior_apply(b), y)
+
+
+@pytest.mark.parametrize("n", SIDES)
+def test_subnormal_fields(plc, n):
+    # P(k) constant: y = 3.125 x.  All of x lies below 2^-1022, whose smallest
+    # unit is 2^-1074; the passes' quantum follows the field down to 2^-1083, so
+    # that their errors stay below a unit; the last rounding adds half a one.
+    # Four allowed (x itself is 2^44 of them).
+    c = plc.Context(n, 5.0 * n, "fp64")
+    k, _ = pk_table_for(n, 5.0 * n)
+    c.set_prior(k, np.full_like(k, 40.0), 0.0, 125.0 / 40.0)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    x = torch.randn((n, n, n), dtype=torch.float64, device="cuda", generator=gen) * 2.0 ** -1030
+    assert 0.0 < float(x.abs().max()) < 2.0 ** -1022
+    off = (c.prior_apply(x) * 2.0 ** 600 - 3.125 * (x * 2.0 ** 600)).abs().max()
+    assert float(off) <= 4.0 * 2.0 ** (600 - 1074)
