@@ -181,6 +181,13 @@ bool run_fixed(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* do
 // Shared memory of the Stockham plane kernel: two planes of up to 108^2 FP32
 // modes.  FP64 planes stay apart: n/2+1 blocks would leave most FP64 pipes idle.
 constexpr size_t kPlaneSmem = 200 * 1024;
+// Sides that take it in a solve or call by itself: public H v 33.3 -> 30.5 us at
+// 72^3, 26.0 -> 21.5 at 48^3.  At 96^3 (where the Stockham schedule has to be
+// asked for) 35.3 -> 37.2, and at 108^3, whose 55 blocks, one to an SM, leave two
+// thirds of the chip idle, 47.5 -> 51.4, a mixed MAP 1847 -> 2000; it pays there
+// beside other solves: two MAPs of 108^3 in a batch 2852 -> 2707 us, sixteen
+// 16.35 -> 15.72 ms.
+constexpr int kPlaneAlone = 72;
 
 // The five passes XF -> YF -> Z -> YI -> XI on the context's stream.
 template <typename T, typename Pro, typename Epi, typename Fin>
@@ -213,7 +220,7 @@ void run_pipeline(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int*
     LaunchScope ls(c, Site(s0 + 0));
     k_xf<T, Pro><<<gx, kThreads, sm, c->stream>>>(pro, A, c->plan, tw, done);
   }
-  if (sizeof(T) == 4 && plane_smem<T>(n) <= kPlaneSmem) {
+  if (sizeof(T) == 4 && plane_smem<T>(n) <= kPlaneSmem && (n <= kPlaneAlone || c->shared_chip)) {
     set_smem4<k_yzy<T>>(kPlaneSmem);
     LaunchScope ls(c, Site(s0 + 2));
     k_yzy<T><<<h, kPlaneThreads, plane_smem<T>(n), c->stream>>>(
