@@ -25,6 +25,9 @@
 // 128^3 / 192^3 / 256^3 went from 327 / 1170 / 3450 us to 88 / 264 / 470.
 #pragma once
 
+#include <cmath>
+#include <vector>
+
 #include "ctx.h"
 #include "fx.cuh"
 #include "passes4.cuh"
@@ -44,6 +47,32 @@ inline FxExps fx_exps(int* p, int n) {
   const size_t h = n / 2 + 1, t = (n + 15) / 16;
   int* b = p + (size_t)n * ((n + 31) / 32);
   return FxExps{p, b, b + h * t, b + 2 * h * t};
+}
+
+// Twiddles W_n^m of the fixed-point passes; empty for lengths without them.
+// long double (at least 64 significant bits on the hosts in use) is software
+// arithmetic on AArch64, so only the first octant is evaluated: creating a
+// context of 256^3 takes 325 us (310 without this table), 498 with all of the
+// circle evaluated, and one of 512^3, which has no such passes, 414 (778).
+inline std::vector<fxw> fx_twiddles(int n) {
+  if (!fixed_length(n)) return {};
+  const int o = n / 8;   // every fixed length is a multiple of 8
+  const long double step = 2.0L * std::acos(-1.0L) / (long double)n;
+  const long double one = (long double)(1ll << kFxOne);
+  std::vector<long long> c(o + 1), s(o + 1);
+  for (int j = 0; j <= o; ++j) {
+    c[j] = std::llrint(std::cos(step * (long double)j) * one);
+    s[j] = std::llrint(std::sin(step * (long double)j) * one);
+  }
+  auto cosine = [&](int m) {   // cos(2 pi m / n) 2^61
+    m = m <= n / 2 ? m : n - m;
+    const int r = m <= n / 4 ? m : n / 2 - m;
+    const long long v = r <= o ? c[r] : s[n / 4 - r];
+    return m <= n / 4 ? v : -v;
+  };
+  std::vector<fxw> tw(n);
+  for (int m = 0; m < n; ++m) tw[m] = fx_factor(cosine(m), -cosine((m + n - n / 4) % n));
+  return tw;
 }
 
 // Resident blocks per SM asked of the compiler: two (up to 128 registers).
