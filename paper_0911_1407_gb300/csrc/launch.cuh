@@ -4,6 +4,7 @@
 #pragma once
 
 #include "ctx.h"
+#include "limits.cuh"
 #include "ops.cuh"
 #include <type_traits>
 
@@ -20,23 +21,13 @@ template <typename T> inline const T* multiplier(const plc_ctx* c);
 template <> inline const float* multiplier<float>(const plc_ctx* c) { return c->M32; }
 template <> inline const double* multiplier<double>(const plc_ctx* c) { return c->M64; }
 
-// Raise a kernel's dynamic shared-memory limit to what the largest grid
-// (n = 512) needs, once per kernel instantiation.
-template <typename T, auto Kernel> inline void set_smem() {
-  static const cudaError_t once = cudaFuncSetAttribute(
-      Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassGeom<T>::smem_bytes_max(512));
-  check(once, "cudaFuncSetAttribute");
+// Dynamic shared memory of the Stockham passes: what the largest grid (n = 512)
+// needs.
+template <typename T, auto Kernel> inline void set_smem(int dev) {
+  set_smem4<Kernel>(dev, PassGeom<T>::smem_bytes_max(512));
 }
 
 inline RedArgs red_args(plc_ctx* c) { return RedArgs{c->partials, c->sc}; }
-
-// Raise a kernel's dynamic shared-memory limit once (also below 48 KB, which
-// is the limit for its static and dynamic shared memory together).
-template <auto Kernel> inline void set_smem4(size_t bytes) {
-  static const cudaError_t once =
-      cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  check(once, "cudaFuncSetAttribute");
-}
 
 // The passes with register four-step line transforms (passes4.cuh) in FP32.
 template <typename T, int N1, int N2, typename Pro, typename Epi, typename Fin>
@@ -50,8 +41,9 @@ void run_pipeline4(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int
   const C* tw = twiddles<T>(c);
   const T* M = m_override ? m_override : multiplier<T>(c);
   const dim3 gx(n / Gm::RY, n), gy(n / Gm::L, h);
-  set_smem4<k4_xf<T, N1, N2, Pro>>(Gm::smem_x);
-  set_smem4<k4_xi<T, N1, N2, Epi, Fin>>(Gm::smem_x);
+  const int dev = current_device();
+  set_smem4<k4_xf<T, N1, N2, Pro>>(dev, Gm::smem_x);
+  set_smem4<k4_xi<T, N1, N2, Epi, Fin>>(dev, Gm::smem_x);
   {
     LaunchScope ls(c, Site(s0 + 0));
     k4_xf<T, N1, N2, Pro><<<gx, kThreads, Gm::smem_x, c->stream>>>(pro, A, tw, done);
@@ -65,16 +57,16 @@ void run_pipeline4(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int
     if constexpr (n <= 128) {
       using Gp = GeoP<N1, N2>;
       constexpr size_t bytes = Gp::template smem<C>();
-      set_smem4<k4_yzy<T, N1, N2>>(bytes);
+      set_smem4<k4_yzy<T, N1, N2>>(dev, bytes);
       LaunchScope ls(c, Site(s0 + 2));
       k4_yzy<T, N1, N2><<<h, Gp::kT, bytes, c->stream>>>(A, M, zero_dc, tw, done);
     }
   };
   auto three_passes = [&]() {
     if constexpr (n > 96) {
-      set_smem4<k4_yf<T, N1, N2>>(Gm::smem_y);
-      set_smem4<k4_z<T, N1, N2>>(Gm::smem_z);
-      set_smem4<k4_yi<T, N1, N2>>(Gm::smem_y);
+      set_smem4<k4_yf<T, N1, N2>>(dev, Gm::smem_y);
+      set_smem4<k4_z<T, N1, N2>>(dev, Gm::smem_z);
+      set_smem4<k4_yi<T, N1, N2>>(dev, Gm::smem_y);
       {
         LaunchScope ls(c, Site(s0 + 1));
         k4_yf<T, N1, N2><<<gy, kThreads, Gm::smem_y, c->stream>>>(A, B, tw, done);
@@ -131,11 +123,12 @@ void run_pipelinex(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int
   const double* M = m_override ? m_override : c->M64;
   const FxExps ex = fx_exps(c->fxexp, n);
   const dim3 gx(n / Gm::RY, n), gy(n / Gm::L, h);
-  set_smem4<kx_xf<N1, N2, Pro>>(Gm::smem_x);
-  set_smem4<kx_yf<N1, N2>>(Gm::smem_y);
-  set_smem4<kx_z<N1, N2>>(Gm::smem_z);
-  set_smem4<kx_yi<N1, N2>>(Gm::smem_y);
-  set_smem4<kx_xi<N1, N2, Epi, Fin>>(Gm::smem_x);
+  const int dev = current_device();
+  set_smem4<kx_xf<N1, N2, Pro>>(dev, Gm::smem_x);
+  set_smem4<kx_yf<N1, N2>>(dev, Gm::smem_y);
+  set_smem4<kx_z<N1, N2>>(dev, Gm::smem_z);
+  set_smem4<kx_yi<N1, N2>>(dev, Gm::smem_y);
+  set_smem4<kx_xi<N1, N2, Epi, Fin>>(dev, Gm::smem_x);
   {
     LaunchScope ls(c, Site(s0 + 0));
     kx_xf<N1, N2, Pro><<<gx, kThreads, Gm::smem_x, c->stream>>>(pro, A, ex, tw, done);
@@ -211,17 +204,18 @@ void run_pipeline(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int*
   cpx<T>* B = static_cast<cpx<T>*>(c->specB);
   const cpx<T>* tw = twiddles<T>(c);
   const dim3 gx((n + G::RY - 1) / G::RY, n), gy((n + G::L - 1) / G::L, h);
-  set_smem<T, k_xf<T, Pro>>();
-  set_smem<T, k_yf<T>>();
-  set_smem<T, k_z<T>>();
-  set_smem<T, k_yi<T>>();
-  set_smem<T, k_xi<T, Epi, Fin>>();
+  const int dev = current_device();
+  set_smem<T, k_xf<T, Pro>>(dev);
+  set_smem<T, k_yf<T>>(dev);
+  set_smem<T, k_z<T>>(dev);
+  set_smem<T, k_yi<T>>(dev);
+  set_smem<T, k_xi<T, Epi, Fin>>(dev);
   {
     LaunchScope ls(c, Site(s0 + 0));
     k_xf<T, Pro><<<gx, kThreads, sm, c->stream>>>(pro, A, c->plan, tw, done);
   }
   if (sizeof(T) == 4 && plane_smem<T>(n) <= kPlaneSmem && (n <= kPlaneAlone || c->shared_chip)) {
-    set_smem4<k_yzy<T>>(kPlaneSmem);
+    set_smem4<k_yzy<T>>(dev, kPlaneSmem);
     LaunchScope ls(c, Site(s0 + 2));
     k_yzy<T><<<h, kPlaneThreads, plane_smem<T>(n), c->stream>>>(
         A, m_override ? m_override : multiplier<T>(c), zero_dc, c->plan, tw, done);
