@@ -101,8 +101,8 @@ void release(plc_ctx* c) {
 
 void ensure_work_fields(plc_ctx* c) {
   const size_t b = sizeof(double) * c->n3();
-  for (int i = 0; i < plc_ctx::kNumWork; ++i)
-    if (!c->wf[i] && (i != plc_ctx::kPrecondField || c->precision == PLC_FP64)) dalloc(&c->wf[i], b);
+  for (void*& p : c->wf)
+    if (!p) dalloc(&p, b);
 }
 
 void ensure_bias_fields(plc_ctx* c) {

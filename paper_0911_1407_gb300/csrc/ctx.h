@@ -115,9 +115,10 @@ struct plc_ctx {
   unsigned long long* hist = nullptr;
 
   // Solver work fields, each n^3 doubles, allocated on first use.
-  // The last one (PLC_FP64 contexts only) holds the Jacobi diagonal M^-1 of
-  // the CG in progress (precond).
-  static constexpr int kNumWork = 14, kPrecondField = 13;
+  // The first holds the FP32 iterate of PLC_MIXED solves, and in PLC_FP64
+  // contexts, whose iterate lives in the caller's buffer, the Jacobi diagonal
+  // M^-1 of the CG in progress (precond).
+  static constexpr int kNumWork = 13, kPrecondField = 0;
   void* wf[kNumWork] = {};
   // Extra work fields of the linear-bias solve, allocated on its first use.
   static constexpr int kNumBiasWork = 12;
