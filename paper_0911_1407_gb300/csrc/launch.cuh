@@ -214,12 +214,17 @@ void run_pipeline(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int*
     LaunchScope ls(c, Site(s0 + 0));
     k_xf<T, Pro><<<gx, kThreads, sm, c->stream>>>(pro, A, c->plan, tw, done);
   }
-  if (sizeof(T) == 4 && plane_smem<T>(n) <= kPlaneSmem && (n <= kPlaneAlone || c->shared_chip)) {
-    set_smem4<k_yzy<T>>(dev, kPlaneSmem);
-    LaunchScope ls(c, Site(s0 + 2));
-    k_yzy<T><<<h, kPlaneThreads, plane_smem<T>(n), c->stream>>>(
-        A, m_override ? m_override : multiplier<T>(c), zero_dc, c->plan, tw, done);
-  } else {
+  bool plane = false;
+  if constexpr (sizeof(T) == 4) {
+    plane = plane_smem<T>(n) <= kPlaneSmem && (n <= kPlaneAlone || c->shared_chip);
+    if (plane) {
+      set_smem4<k_yzy<T>>(dev, kPlaneSmem);
+      LaunchScope ls(c, Site(s0 + 2));
+      k_yzy<T><<<h, kPlaneThreads, plane_smem<T>(n), c->stream>>>(
+          A, m_override ? m_override : multiplier<T>(c), zero_dc, c->plan, tw, done);
+    }
+  }
+  if (!plane) {
     {
       LaunchScope ls(c, Site(s0 + 1));
       k_yf<T><<<gy, kThreads, sm, c->stream>>>(A, B, c->plan, tw, done);
@@ -381,7 +386,7 @@ template <typename TC> void cg_update(plc_ctx* c, TC* x, TC* r, const TC* p, con
                                       const LoopCtl& loop) {
   // one wave (FP32: 4 blocks of 256 per SM at its 56 registers, 73.8 us
   // against 77.1 with two waves at 256^3)
-    const int nb = pointwise_blocks((long long)c->n3(), c->sms, sizeof(TC) == 8 ? 3 : 4);
+  const int nb = pointwise_blocks((long long)c->n3(), c->sms, sizeof(TC) == 8 ? 3 : 4);
   LaunchScope ls(c, sizeof(TC) == 4 ? S_CG_UPDATE32 : S_CG_UPDATE64);
   if (jac)
     k_cg_update<TC, true><<<nb, kThreads, 0, c->stream>>>(x, r, p, Hp, precond_field<TC>(c, D),

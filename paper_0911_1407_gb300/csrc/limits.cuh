@@ -21,7 +21,7 @@ inline int current_device() {
 // at their first launch) does no harm.
 template <auto Kernel> inline void set_smem4(int dev, size_t bytes) {
   constexpr int kMaxDevices = 64;
-  static std::atomic<bool> set[kMaxDevices];
+  static std::atomic<bool> set[kMaxDevices] = {};
   if (dev < kMaxDevices && set[dev].load(std::memory_order_acquire)) return;
   check(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
         "cudaFuncSetAttribute");
