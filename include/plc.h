@@ -273,8 +273,9 @@ plc_status plc_compare(plc_ctx* ctx, const double* a, const double* b, double* r
  * 5 and 10 Mpc/h before the matter statistics): y = x convolved with a
  * normalised Gaussian of radius `radius` (Mpc/h, >= 0), i.e. every Fourier
  * mode multiplied by exp(-|k|^2 radius^2 / 2), |k| as for the prior.  x, y:
- * double fields (may alias).  Transforms in 64-bit block fixed point for
- * lengths with a four-step schedule, FP64 otherwise; uses the solver work
+ * double fields (may alias).  Transforms in 64-bit block fixed point for n =
+ * 32, 64, 96, 128, 192 and 256 (unless the Stockham schedule is set, see
+ * plc_set_fft_schedule), FP64 otherwise; uses the solver work
  * fields as scratch.  Needs no prior.  Synchronises the stream. */
 plc_status plc_smooth(plc_ctx* ctx, const double* x, double* y, double radius);
 
@@ -296,9 +297,11 @@ plc_status plc_log_stats(plc_ctx* ctx, const double* delta, double lo, double wi
 /* FFT schedule of the transforms (an aid to performance, the paper has no
  * counterpart).  A length n = f1 f2 with a register four-step form can run
  * its FP32 transforms with the factors (f1, f2) or with the shared-memory
- * Stockham stages (f1 = f2 = 0); FP64 fields run in 64-bit block fixed point
- * (whichever factors are set) or, at f1 = f2 = 0, in the FP64 Stockham
- * stages.  Every schedule computes the same transform.  plc_set_fft_schedule selects one (INVALID_ARG if (f1, f2)
+ * Stockham stages (f1 = f2 = 0).  FP64 fields of n = 32, 64, 96, 128, 192 and
+ * 256 run in 64-bit block fixed point, whichever factors are set, and at f1 =
+ * f2 = 0 in the FP64 Stockham stages; those of every other n, 512 among them,
+ * always in the FP64 Stockham stages.  Every schedule computes the same
+ * transform.  plc_set_fft_schedule selects one (INVALID_ARG if (f1, f2)
  * is not offered for this n).  plc_autotune times `reps` (1..1000)
  * Hessian-vector products with each schedule offered for n, keeps the
  * fastest and returns it (f1, f2 and its time per Hv in microseconds, any

@@ -394,8 +394,9 @@ void bias_cg_hv(plc_ctx* c, const TC* r, const TC* Dj, TC* p, const TC* E, const
   const int* done = &c->sc->done;
   const TC* Mb = bias_multiplier<TC>(c);
   if (jac)
-    run_pipeline<TC>(c, ProCgDirE<TC, true>{{r, precond_field<TC>(c, Dj), (TC)c->jac_c, p, c->sc}, E}, EpiMul<TC>{Q, t},
-                     FinNone{}, 0, done, kBiasSites, Mb);
+    run_pipeline<TC>(c,
+                     ProCgDirE<TC, true>{{r, precond_field<TC>(c, Dj), (TC)c->jac_c, p, c->sc}, E},
+                     EpiMul<TC>{Q, t}, FinNone{}, 0, done, kBiasSites, Mb);
   else
     run_pipeline<TC>(c, ProCgDirE<TC, false>{{r, Dj, (TC)c->jac_c, p, c->sc}, E},
                      EpiMul<TC>{Q, t}, FinNone{}, 0, done, kBiasSites, Mb);

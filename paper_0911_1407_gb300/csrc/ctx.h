@@ -37,9 +37,9 @@ extern const char* const kSiteNames[S_NSITES];
 
 // Line-transform schedules with a register four-step form: n = f1 f2
 // (passes4.cuh in FP32; passesx.cuh for FP64 fields of a fixed_length, which
-// takes the first entry of its n whichever is set).  The first entry for an n is the default;
-// plc_autotune times every FP32 entry for n and the Stockham form
-// (f1 = f2 = 0).
+// takes the first entry of its n whichever is set).  The first entry for an n
+// is the default; plc_autotune times every FP32 entry for n and the Stockham
+// form (f1 = f2 = 0).
 struct FourStepShape {
   int n, f1, f2;
 };
@@ -161,8 +161,8 @@ void grad_newton(plc_ctx* c, const TS* s, const double* w, const int32_t* N, dou
                  T* g, TC* D, TC* r, bool jac);
 // Newton trial point s + tau xi without an FFT (see k_newton_update).
 // The sums of the FP64 gradient of the mixed solve at s (fixed-point
-// transforms, no field stored) into sc->red; false when the length has no
-// four-step schedule (nothing launched).
+// transforms, no field stored) into sc->red; false (nothing launched) when the
+// length has no fixed-point passes or the schedule is the Stockham stages.
 bool grad_sums_ff(plc_ctx* c, const double* s, const double* w, const int32_t* N, double nbar,
                   bool jac);
 template <typename T, typename TC>

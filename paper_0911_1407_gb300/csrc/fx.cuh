@@ -11,9 +11,13 @@
 // E is chosen per tile from the data, by the L1 norm of its lines: every
 // intermediate of a DFT of a line is a partial sum of its elements times unit
 // factors, so |re|, |im| <= L1 throughout and L1 < 2^62 quanta rules out
-// overflow.  The quantum is then at most 2^-61 L1 <= 2^-61 sqrt(2) N rms, and
-// for N = 256 its rounding error is about 2^-54.5 of the line's rms, below
-// the 2^-53 relative rounding of each FP64 butterfly it replaces.
+// overflow.  The quantum is at most 2^-61 of the largest L1 norm among the
+// tile's 16 lines.  For a line that reaches it, L1 <= sqrt(2) N rms makes the
+// rounding error about 2^-54.5 of its rms at N = 256, below the 2^-53 relative
+// rounding of each FP64 butterfly it replaces.  For the others the error is the
+// same absolute one: a line 2^k times smaller has it 2^k times larger beside
+// itself, where the butterflies' would shrink with the line; the transform
+// across the lines then adds either to the larger ones.
 #pragma once
 
 #include "common.cuh"

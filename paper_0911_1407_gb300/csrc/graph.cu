@@ -3,8 +3,9 @@
 // The host driver (solver.cu) reads the device scalars after every gradient,
 // CG chunk and line-search trial to take its decisions.  Here the same
 // decisions are taken by one-thread control kernels, or by the last block of
-// the loop's own kernel, that read the device scalars and set the conditions of CUDA graph conditional nodes, so that a
-// whole solve is one graph launch with no host round trip:
+// the loop's own kernel, that read the device scalars and set the conditions of
+// CUDA graph conditional nodes, so that a whole solve is one graph launch with
+// no host round trip:
 //
 //   init:  [PLC_MIXED: s -> FP32]  FFT gradient  ctl_init
 //   WHILE newton:
@@ -414,8 +415,8 @@ void capture_solve(plc_ctx* c, cudaGraph_t top, const std::vector<cudaStream_t>&
   // a conditional node for the graph to instantiate)
   const int first = o.start == 0 ? 0 : (o.g0_norm > 0.0 ? 2 : (o.start == 2 ? 3 : 1));
   if (first == 1) mk(&h_first);
-  // the switch's sums-only check: mixed solves of lengths with fixed-point
-  // transforms (a four-step schedule)
+  // the switch's sums-only check: mixed solves that run the fixed-point
+  // transforms (see run_fixed)
   bool has_check = false;
   if constexpr (kMixed) has_check = c->plan.f1 != 0 && fixed_length(c->n);
   if (has_check) {

@@ -51,8 +51,10 @@ void run_pipeline4(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int
   // The y and z passes of a plane in one block (k4_yzy) up to 96^3: mixed MAP
   // at 32^3 904 -> 835 us, 64^3 867 -> 832, 96^3 1240 -> 1237.  At 128^3 its 65
   // planes leave half the chip idle, and a solve by itself is slower (1601 ->
-  // 1645 us), but solves that share the chip gain from the traffic saved
-  // (64 mocks up to 128^3: 37.8 -> 36.2 ms).
+  // 1645 us), but solves that share the chip gain from the traffic saved, two
+  // of them already: batches of 2, 4, 8 and 16 MAPs of 128^3 2233 -> 2157, 3618
+  // -> 3447, 7567 -> 7038 and 15020 -> 14110 us; 64 mocks up to 128^3 37.8 ->
+  // 36.2 ms.
   auto fused = [&]() {
     if constexpr (n <= 128) {
       using Gp = GeoP<N1, N2>;
@@ -153,9 +155,9 @@ void run_pipelinex(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int
   check(cudaGetLastError(), "spectral pipeline launch");
 }
 
-// False when the context's schedule is the Stockham stages (run_pipeline then
-// takes the FP64 Stockham passes); any four-step schedule runs the default
-// factors of its length.
+// False when the length has no fixed-point passes or the context's schedule is
+// the Stockham stages (run_pipeline then takes the FP64 Stockham passes); any
+// four-step schedule of the others runs the default factors of its length.
 template <typename Pro, typename Epi, typename Fin>
 bool run_fixed(plc_ctx* c, Pro pro, Epi epi, Fin fin, int zero_dc, const int* done, int s0,
                const double* m_override) {
@@ -268,7 +270,7 @@ void grad_newton(plc_ctx* c, const TS* s, const double* w, const int32_t* N, dou
                  T* g, TC* D, TC* r, bool jac) {
   if constexpr (std::is_same<T, double>::value && std::is_same<TC, float>::value) {
     // the FP64 gradient of the mixed solve: fixed-point transforms and a
-    // float-float epilogue where the length has a four-step schedule
+    // float-float epilogue where the length has fixed-point passes
     const EpiGradFF<true> epi{s, w, N, ff(nbar), ff(c->mu), y, g, D, r, (float)c->jac_c,
                               jac ? 1 : 0, static_cast<const ff*>(c->expff)};
     if (run_fixed(c, ProShift<double, double>{s, c->mu}, epi, FinGrad<6>{}, 0, nullptr, S_GXFF,
@@ -286,7 +288,7 @@ void grad_newton(plc_ctx* c, const TS* s, const double* w, const int32_t* N, dou
 // same pipeline with nothing stored: the sums of -ln P and ||g||^2 into
 // sc->red, FinGrad), for a stopping test that may end the solve before the
 // gradient's fields are needed.  False (nothing run)
-// when the length has no four-step schedule.
+// where run_fixed has none.
 inline bool grad_sums_ff_impl(plc_ctx* c, const double* s, const double* w, const int32_t* N,
                               double nbar, bool jac) {
   const EpiGradFF<false> epi{s, w, N, ff(nbar), ff(c->mu), nullptr, nullptr, nullptr, nullptr,

@@ -1,13 +1,14 @@
 // log64.cuh -- ln u of a double on the integer pipes (see exp64.cuh).
 //
-// Table-driven: u = 2^e m, m in [1, 2); c an 11-bit reciprocal of m's 1/128
-// interval, r = m c / 1024 - 1 exactly (|r| <= 2^-7), ln u = e ln2 -
-// ln(c / 1024) + ln(1 + r), the last by its series to degree 8 (remainder
-// below 2^-66), in fixed point.  The intervals next to u = 1 on both sides have
-// c / 1024 a power of two, so that ln u = ln(1 + r) there and keeps its
-// relative accuracy down to |r| = 2^-14.  Error below 2^-59 for |ln u| < 3 and
-// 2^-55 for |ln u| < 31 before the rounding to 53 bits.  Nearer to 1, and
-// for u <= 0, subnormal, infinite, NaN or outside 2^+-44: the library function.
+// Table-driven as in Tang (ACM TOMS 16, 1990), with a reciprocal in place of
+// the quotient that reduces the argument: u = 2^e m, m in [1, 2); c an 11-bit
+// reciprocal of m's 1/128 interval, r = m c / 1024 - 1 exactly (|r| <= 2^-7),
+// ln u = e ln2 - ln(c / 1024) + ln(1 + r), the last by its series to degree 8
+// (remainder below 2^-66), in fixed point.  The intervals next to u = 1 on both
+// sides have c / 1024 a power of two, so that ln u = ln(1 + r) there and keeps
+// its relative accuracy down to |r| = 2^-14.  Error below 2^-59 for |ln u| < 3
+// and 2^-55 for |ln u| < 31 before the rounding to 53 bits.  Nearer to 1, and for
+// u <= 0, subnormal, infinite, NaN or outside 2^+-44: the library function.
 #pragma once
 
 #include "exp64.cuh"

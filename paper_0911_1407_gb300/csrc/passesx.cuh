@@ -16,8 +16,11 @@
 //   XI  A, EC -> doubles for the epilogue
 //
 // A tile that meets a NaN or an infinity marks its exponent (kFxNaN), which
-// every later tile it reaches inherits, and the epilogue then sees NaN: a
-// transform spreads such a value over the whole grid in any arithmetic.
+// every later tile it reaches inherits, and the epilogue then sees NaN in every
+// cell: a transform spreads such a value over the whole grid in any arithmetic
+// (the FP64 passes give a mixture of NaNs and infinities).  Multipliers must not
+// be negative (kx_z reads a sign bit as part of the exponent; the prior's, the
+// bias's and the smoothing's are not), and subnormal ones count as zero.
 //
 // What bounds them: the FP64 Stockham passes they replace ran at 0.74-0.8 of
 // the FP64 pipe (2 per SM and clock).  These issue on half of all cycles with

@@ -112,7 +112,7 @@ struct Lognormal {
                        T* y, T* g, TC* D, TC* r, bool jac) {
     grad_newton<T, TS, TC>(c, s, w, N, nbar, y, g, D, r, jac);
   }
-  // the sums of the FP64 gradient alone (false: not offered for this length)
+  // the sums of the FP64 gradient alone (false: not offered, see grad_sums_ff)
   static bool gradient_sums(plc_ctx* c, const double* s, const double* w, const int32_t* N,
                             double nbar, bool jac) {
     return grad_sums_ff(c, s, w, N, nbar, jac);
