@@ -88,7 +88,7 @@ template <typename T> void dalloc(T** p, size_t bytes) {
 void release(plc_ctx* c) {
   plc::graph_release(c);
   plc::profile_release(c);
-  void* ptrs[] = {c->specA, c->specB, c->tables, c->M64, c->M32,
+  void* ptrs[] = {c->specA, c->specB, c->tw64, c->tw32, c->twfx, c->fxexp, c->expff, c->M64, c->M32,
                   c->lk, c->lP, c->sc, c->partials, c->Mb64, c->Mb32, c->lkb, c->lbb, c->hist};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -224,43 +224,43 @@ plc_status plc_create(plc_ctx** out, int n, double box, int precision, void* str
     const size_t spec = sizeof(double2) * h * n * n;
     dalloc(&c->specA, spec);
     dalloc(&c->specB, spec);
+    // small buffers one by one: the tables in one block saved 10 us here, but the
+    // kernels of small solves felt where the buffers behind them came to lie (FP64
+    // MAP at 32^3: 861 us as it is, 873 with the tile exponents in that block, 898
+    // with them apart)
+    dalloc(&c->tw64, sizeof(double2) * n);
+    dalloc(&c->tw32, sizeof(float2) * n);
+    const std::vector<plc::fxw> tfx = plc::fx_twiddles(n);
+    if (!tfx.empty()) {
+      dalloc(&c->twfx, sizeof(plc::fxw) * n);
+      dalloc(&c->fxexp, sizeof(int) * plc::fx_exps_ints(n));
+    }
+    dalloc(&c->expff, sizeof(float2) * 64);
     dalloc(&c->sc, sizeof(plc::DevScalars));
     plc::check(cudaMallocHost(reinterpret_cast<void**>(&c->sc_host), sizeof(plc::DevScalars)),
                "cudaMallocHost");
     const size_t xi_blocks = (size_t)((n + 15) / 16) * n;
     c->partial_blocks = std::max(xi_blocks, (size_t)c->sms * 8);
     dalloc(&c->partials, sizeof(double) * plc::kMaxRed * c->partial_blocks);
-    // the constant tables, in one block and one copy: twiddles W_n^m =
-    // exp(-2 pi i m / n) from the FP64 host sin/cos, 2^(j/64), j < 64, in
-    // float-float (the table of the float-float exp), the fixed-point twiddles
-    // and, behind what is copied, room for the fixed-point tile exponents
-    const std::vector<plc::fxw> tfx = plc::fx_twiddles(n);
-    const size_t off32 = sizeof(double2) * n, offe = off32 + sizeof(float2) * n;
-    const size_t offx = (offe + sizeof(float2) * 64 + 15) / 16 * 16;
-    const size_t copied = offx + sizeof(plc::fxw) * tfx.size();
-    dalloc(&c->tables, copied + (tfx.empty() ? 0 : sizeof(int) * plc::fx_exps_ints(n)));
-    std::vector<double2> tab((copied + sizeof(double2) - 1) / sizeof(double2));
-    char *const th = reinterpret_cast<char*>(tab.data()), *const td = static_cast<char*>(c->tables);
-    double2* const t64 = tab.data();
-    float2 *const t32 = reinterpret_cast<float2*>(th + off32), *const e2 = reinterpret_cast<float2*>(th + offe);
+    // twiddles W_n^m = exp(-2 pi i m / n), from the FP64 host sin/cos
+    std::vector<double2> t64(n);
+    std::vector<float2> t32(n);
     for (int m = 0; m < n; ++m) {
       const double ang = 2.0 * M_PI * (double)m / (double)n;
       t64[m] = make_double2(std::cos(ang), -std::sin(ang));
       t32[m] = make_float2((float)t64[m].x, (float)t64[m].y);
     }
+    plc::check(cudaMemcpyAsync(c->tw64, t64.data(), sizeof(double2) * n, cudaMemcpyHostToDevice, c->stream), "copy twiddles");
+    plc::check(cudaMemcpyAsync(c->tw32, t32.data(), sizeof(float2) * n, cudaMemcpyHostToDevice, c->stream), "copy twiddles");
+    if (!tfx.empty())
+      plc::check(cudaMemcpyAsync(c->twfx, tfx.data(), sizeof(plc::fxw) * n, cudaMemcpyHostToDevice, c->stream), "copy twiddles");
+    // 2^(j/64), j < 64, in float-float (the table of the float-float exp)
+    std::vector<float2> e2(64);
     for (int j = 0; j < 64; ++j) {
       const double v = std::exp2((double)j / 64.0);
       e2[j] = make_float2((float)v, (float)(v - (double)(float)v));
     }
-    if (!tfx.empty()) {
-      std::memcpy(th + offx, tfx.data(), sizeof(plc::fxw) * tfx.size());
-      c->twfx = td + offx;
-      c->fxexp = reinterpret_cast<int*>(td + copied);
-    }
-    c->tw64 = reinterpret_cast<double2*>(td);
-    c->tw32 = reinterpret_cast<float2*>(td + off32);
-    c->expff = td + offe;
-    plc::check(cudaMemcpyAsync(c->tables, th, copied, cudaMemcpyHostToDevice, c->stream), "copy tables");
+    plc::check(cudaMemcpyAsync(c->expff, e2.data(), sizeof(float2) * 64, cudaMemcpyHostToDevice, c->stream), "copy exp table");
     plc::check(cudaMemsetAsync(c->sc, 0, sizeof(plc::DevScalars), c->stream), "clear scalars");
     plc::check(cudaStreamSynchronize(c->stream), "stream synchronize");
     return PLC_OK;

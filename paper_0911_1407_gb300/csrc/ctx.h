@@ -74,7 +74,6 @@ struct plc_ctx {
   // FFT scratch: two half-spectra sized for double2 (float2 reuses them).
   void* specA = nullptr;
   void* specB = nullptr;
-  void* tables = nullptr;      // block of the constant tables that the next five point into
   double2* tw64 = nullptr;
   float2* tw32 = nullptr;
   void* twfx = nullptr;        // fixed-point twiddles (fxw, fx.cuh); fixed_length(n) only

@@ -55,8 +55,8 @@ inline FxExps fx_exps(int* p, int n) {
 // Twiddles W_n^m of the fixed-point passes; empty for lengths without them.
 // long double (at least 64 significant bits on the hosts in use) is software
 // arithmetic on AArch64, so only the first octant is evaluated: creating a
-// context of 256^3 takes 325 us (310 without this table), 498 with all of the
-// circle evaluated, and one of 512^3, which has no such passes, 414 (778).
+// context of 256^3 takes 338 us (310 without this table), 490 with all of the
+// circle evaluated, and one of 512^3, which has no such passes, 420 (778).
 inline std::vector<fxw> fx_twiddles(int n) {
   if (!fixed_length(n)) return {};
   const int o = n / 8;   // every fixed length is a multiple of 8
