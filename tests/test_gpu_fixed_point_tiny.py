@@ -1,9 +1,9 @@
 """Values far below the quantum of the fixed-point FP64 passes: they count as
-nothing, not as one quantum of a fixed sign.
+nothing, not as one quantum of a fixed sign (and fields of subnormals, which have
+a quantum of their own, keep their value).
 
-The fields are chosen so that the passes are exact, or round once in a place
-that can be named, where one quantum too many in each of a line's elements
-shows.
+Bars.  The fields are chosen so that the passes are exact or round in one known
+place; an error of one quantum in every element of a line then shows.
 """
 import numpy as np
 import pytest
